@@ -245,8 +245,8 @@ struct LineTables {
     float* us_lncdf;    // [kUsNx * kUsNu]
     unsigned char* us_guide;  // [kUsNx * kGuideN]
     float* rtab;        // [kRtabElems]
-    float4* rquad;      // [kRquadElems] (built with rtab)
-    double* work;       // scratch: Weideman coefficients + R-table masses
+    float4* rquad;      // [kRquadElems] (built with rtab; scratch of its build before that)
+    double* work;       // scratch of the builds, line_tables_work_doubles() long
 };
 size_t line_tables_work_doubles();
 cudaError_t build_line_tables(double a, const LineTables& T, bool with_r, cudaStream_t s);

@@ -22,20 +22,41 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 
-// Fourier coefficients of Weideman's expansion, one thread per coefficient.
-__global__ void k_weideman(double* c, int N, double L)
+// FP64 issues one warp instruction in 16 cycles on this part (2 lanes per
+// clock and SM), so the builds below are bound by the FP64 pipes they keep
+// busy: each spreads its transcendental work over all SMs in small blocks and
+// leaves only the sums, whose order fixes the tables' last bits, to one
+// thread: 0.09 ms without the R table, 1.6 ms before.
+
+// Fourier coefficients of Weideman's expansion: one block per coefficient,
+// the trapezoidal terms in parallel, added in index order by one thread.
+// 520 us as one 48-thread block that evaluated the terms serially.
+constexpr int kWeidemanTerms = 4 * kWeidemanN - 1;
+constexpr int kCoefBlock = 64;
+
+__device__ void weideman_block(double* c, int N, double L, int n)
 {
-    int n = blockIdx.x * blockDim.x + threadIdx.x + 1;
-    if (n > N) return;
+    __shared__ double f[kWeidemanTerms], cs[kWeidemanTerms];
     const int M = 2 * N;
-    double s = 0.0;
-    for (int k = -M + 1; k <= M - 1; ++k) {
+    for (int q = threadIdx.x; q < kWeidemanTerms; q += blockDim.x) {
+        const int k = q - M + 1;
         double th = k * kPi / M;
         double t = L * tan(0.5 * th);
-        s += (L * L + t * t) * exp(-t * t) * cos(n * th);
+        f[q] = (L * L + t * t) * exp(-t * t);
+        cs[q] = cos(n * th);
     }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double s = 0.0;
+    for (int q = 0; q < kWeidemanTerms; ++q) s += f[q] * cs[q];
     c[n - 1] = s / (2.0 * M);
 }
+
+__global__ void k_weideman(double* c, int N, double L) { weideman_block(c, N, L, (int)blockIdx.x + 1); }
+
+// One-warp blocks: the slice's 5000 nodes then reach every SM's FP64 pipe
+// (493 us as 20 blocks of 256).
+constexpr int kVoigtBlock = 32;
 
 __global__ void k_voigt(double a, const double* c, int N, double L, float* lnH, float* H0)
 {
@@ -93,63 +114,99 @@ __device__ double us_xnode(int i)
     return i < 18 ? 8.0 * i / 18.0 : 8.0 * pow(37.5, (i - 18) / 21.0);
 }
 
-// One thread per sampler row: sequential cumulative sum, then ln CDF and
-// the row's search guide.
-// One block per row: the cell masses in parallel, then the normalisation
-// and running sums by one thread in index order (the same sums, in the same
-// order, as a serial build), the logs in parallel, the guide by one thread.
-__global__ void k_usampler(double a, float* xs, float* lncdf, unsigned char* guide)
+// First stage of a line's tables, all independent of one another: blocks
+// [0, N) one Weideman coefficient each; then the sampler rows' cell masses,
+// the ln sigmoid of the guide bins' left edges, and (with_r) the cell masses
+// at the R table's |x| nodes, one value per thread.
+constexpr int kUsMasses = kUsNx * (kUsNu - 1);
+constexpr int kRMasses = kRnX * (kUsNu - 1);
+
+__global__ void __launch_bounds__(kCoefBlock) k_line_stage1(double a, double* coef, int N, double L, double* us_mass,
+                                                            double* guide_lt, double* r_mass)
 {
-    __shared__ double mass[kUsNu - 1];
-    __shared__ double cdf[kUsNu];
-    const int i = blockIdx.x;
-    const double x = us_xnode(i);
-    for (int j = threadIdx.x; j < kUsNu - 1; j += blockDim.x) mass[j] = cell_mass(x, a, j);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        xs[i] = (float)x;
-        double tot = 0.0;
-        for (int j = 0; j < kUsNu - 1; ++j) tot += mass[j];
-        double run = 0.0;
-        cdf[0] = 0.0;
-        for (int j = 1; j < kUsNu; ++j) {
-            run += mass[j - 1];
-            cdf[j] = run / tot;
-        }
+    if ((int)blockIdx.x < N) {
+        weideman_block(coef, N, L, (int)blockIdx.x + 1);
+        return;
     }
-    __syncthreads();
-    float* row = lncdf + (size_t)i * kUsNu;
-    for (int j = threadIdx.x; j < kUsNu; j += blockDim.x) {
-        const double C = cdf[j];
-        row[j] = (float)log(j > 0 && C > kUsFloor ? C : kUsFloor);
+    int e = ((int)blockIdx.x - N) * kCoefBlock + (int)threadIdx.x;
+    if (e < kUsMasses) {
+        us_mass[e] = cell_mass(us_xnode(e / (kUsNu - 1)), a, e % (kUsNu - 1));
+        return;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned char* gd = guide + (size_t)i * kGuideN;
-        int j = 0;
-        for (int m = 0; m < kGuideN; ++m) {
-            double w = -kGuideW + 2.0 * kGuideW * m / kGuideN;
-            double lt = -log1p(exp(-w));          // ln sigmoid(w)
-            while (j < kUsNu - 2 && (double)row[j + 1] <= lt) ++j;
-            gd[m] = (unsigned char)j;
-        }
+    e -= kUsMasses;
+    if (e < kGuideN) {
+        const double w = -kGuideW + 2.0 * kGuideW * e / kGuideN;
+        guide_lt[e] = -log1p(exp(-w));          // ln sigmoid(w)
+        return;
+    }
+    e -= kGuideN;
+    if (r_mass && e < kRMasses) {
+        double x = kRxMax * (e / (kUsNu - 1)) / (kRnX - 1);
+        r_mass[e] = cell_mass(x, a, e % (kUsNu - 1));
     }
 }
 
-// Normalised sampler masses at the R-table |x| nodes: p[jx][k].
-__global__ void k_rmasses(double a, double* p)
+// One block per sampler row: the running sums of the cell masses by one
+// thread in index order (the last one is the row's total), then the
+// normalised CDF's logs and the guide in parallel. The masses are positive
+// (the expansion of exp(-u^2) over a cell is), so the row does not decrease
+// and a guide entry, the largest node j <= kUsNu - 2 with row[j] <= lt, is
+// found by bisection. 545 us when one thread also divided and built the
+// guide.
+__global__ void __launch_bounds__(256) k_usampler(const double* us_mass, const double* guide_lt, float* xs,
+                                                  float* lncdf, unsigned char* guide)
 {
-    int jx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (jx >= kRnX) return;
-    double x = kRxMax * jx / (kRnX - 1);
-    double* row = p + (size_t)jx * (kUsNu - 1);
-    double tot = 0.0;
-    for (int k = 0; k < kUsNu - 1; ++k) {
-        double m = cell_mass(x, a, k);
-        row[k] = m;
-        tot += m;
+    __shared__ double run[kUsNu];
+    __shared__ float row[kUsNu];
+    const int i = blockIdx.x;
+    for (int j = threadIdx.x; j < kUsNu - 1; j += blockDim.x) run[j + 1] = us_mass[i * (kUsNu - 1) + j];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        xs[i] = (float)us_xnode(i);
+        double s = 0.0;
+        run[0] = 0.0;
+        for (int j = 1; j < kUsNu; ++j) {
+            s += run[j];
+            run[j] = s;
+        }
     }
-    for (int k = 0; k < kUsNu - 1; ++k) row[k] /= tot;
+    __syncthreads();
+    const double tot = run[kUsNu - 1];
+    for (int j = threadIdx.x; j < kUsNu; j += blockDim.x) {
+        const double C = run[j] / tot;
+        const float v = (float)log(j > 0 && C > kUsFloor ? C : kUsFloor);
+        row[j] = v;
+        lncdf[(size_t)i * kUsNu + j] = v;
+    }
+    __syncthreads();
+    for (int m = threadIdx.x; m < kGuideN; m += blockDim.x) {
+        const double lt = guide_lt[m];
+        int lo = 0, hi = kUsNu - 2;             // row[lo] <= lt or lo = 0; row[hi + 1] > lt or hi = kUsNu - 2
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((double)row[mid] <= lt) lo = mid;
+            else hi = mid - 1;
+        }
+        guide[(size_t)i * kGuideN + m] = (unsigned char)lo;
+    }
+}
+
+// Normalises the masses at one R-table |x| node in place (one block per
+// node; the total in index order by one thread).
+__global__ void __launch_bounds__(256) k_rnorm(double* p)
+{
+    __shared__ double m[kUsNu - 1];
+    __shared__ double tot;
+    double* row = p + (size_t)blockIdx.x * (kUsNu - 1);
+    for (int k = threadIdx.x; k < kUsNu - 1; k += blockDim.x) m[k] = row[k];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int k = 0; k < kUsNu - 1; ++k) s += m[k];
+        tot = s;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < kUsNu - 1; k += blockDim.x) row[k] = m[k] / tot;
 }
 
 // rquad(k, j, i) = the R table's four (g, x) corners of cell (k, j) at Delta_i.
@@ -164,31 +221,72 @@ __global__ void k_rquad(const float* rtab, float4* rquad)
     rquad[e] = make_float4(r00[0], r00[kRnD], r00[(size_t)kRnX * kRnD], r00[(size_t)kRnX * kRnD + kRnD]);
 }
 
-// R(D_i; x_j, g_k) = sum_c p_c G(D_i - m_c (g_k - 1); s_k), one thread per entry.
-__global__ void k_rtable(const double* p, float* rtab)
+// R(D_i; x_j, g_k) = sum_c p_c(x_j) G(D_i - m_c (g_k - 1); s_k). The Gaussian
+// depends on (k, c, i) only, so it is tabulated first (2.0e6 exponentials
+// instead of 4.0e8, one per table entry and sampler cell) and the table is a
+// product of [x_j][c] with [c][D_i] for each g_k: 4.0e8 FP64 multiply-adds,
+// 0.64 ms at the FP64 pipes' rate. Measured 0.15 ms (kernel) + 0.79 ms
+// (product); 19.9 ms with the exponential in the sum. The sum runs over c in
+// index order, as a serial sum would.
+struct RNode {
+    double gm1, inv2s2, norm;
+};
+
+__device__ __forceinline__ RNode r_node(int kg)
 {
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= kRtabElems) return;
-    int i = (int)(e % kRnD);
-    int jx = (int)((e / kRnD) % kRnX);
-    int kg = (int)(e / ((size_t)kRnD * kRnX));
-    double D = -kRdMax + kRdStep * i;
     double g = -1.0 + 2.0 * kg / (kRnG - 1);
     double sg = sqrt(fmax(0.0, 1.0 - g * g)) / sqrt(2.0);
     double s = sg > kRsMin ? sg : kRsMin;
-    double inv2s2 = 0.5 / (s * s);
-    double norm = 1.0 / (sqrt(2.0 * kPi) * s);
-    const double* row = p + (size_t)jx * (kUsNu - 1);
-    double acc = 0.0;
-    for (int c = 0; c < kUsNu - 1; ++c) {
-        double lo = unode(c);
-        double hi = unode(c + 1);
-        double m = 0.5 * (lo + hi);
-        double y = D - m * (g - 1.0);
-        acc += row[c] * exp(-y * y * inv2s2);
-    }
-    rtab[e] = (float)(acc * norm);
+    return RNode{g - 1.0, 0.5 / (s * s), 1.0 / (sqrt(2.0 * kPi) * s)};
 }
+
+constexpr size_t kRkernElems = (size_t)kRnG * (kUsNu - 1) * kRnD;
+
+// kern[k][c][i] = exp(-y^2 / (2 s_k^2)); one block per (c, k).
+__global__ void __launch_bounds__(224) k_rkernel(double* kern)
+{
+    const int c = blockIdx.x, kg = blockIdx.y, i = threadIdx.x;
+    __shared__ RNode sn;
+    if (threadIdx.x == 0) sn = r_node(kg);
+    __syncthreads();
+    if (i >= kRnD) return;
+    const RNode nd = sn;
+    double D = -kRdMax + kRdStep * i;
+    double lo = unode(c);
+    double hi = unode(c + 1);
+    double m = 0.5 * (lo + hi);
+    double y = D - m * nd.gm1;
+    kern[((size_t)kg * (kUsNu - 1) + c) * kRnD + i] = exp(-y * y * nd.inv2s2);
+}
+
+// One block per (kRtJ nodes x_j, g_k), one thread per D_i: each kernel value
+// is read once for kRtJ sums. 40 x 25 blocks of 7 warps, all resident.
+constexpr int kRtJ = 8;
+
+__global__ void __launch_bounds__(224) k_rtable(const double* p, const double* kern, float* rtab)
+{
+    const int j0 = blockIdx.x * kRtJ, kg = blockIdx.y, i = threadIdx.x;
+    __shared__ double sp[kRtJ][kUsNu - 1];
+    __shared__ double norm;
+    for (int q = threadIdx.x; q < kRtJ * (kUsNu - 1); q += blockDim.x)
+        sp[q / (kUsNu - 1)][q % (kUsNu - 1)] = p[(size_t)j0 * (kUsNu - 1) + q];
+    if (threadIdx.x == 0) norm = r_node(kg).norm;
+    __syncthreads();
+    if (i >= kRnD) return;
+    const double* e = kern + (size_t)kg * (kUsNu - 1) * kRnD + i;
+    double acc[kRtJ];
+#pragma unroll
+    for (int j = 0; j < kRtJ; ++j) acc[j] = 0.0;
+    for (int c = 0; c < kUsNu - 1; ++c) {
+        const double v = e[(size_t)c * kRnD];
+#pragma unroll
+        for (int j = 0; j < kRtJ; ++j) acc[j] += sp[j][c] * v;
+    }
+#pragma unroll
+    for (int j = 0; j < kRtJ; ++j) rtab[((size_t)kg * kRnX + j0 + j) * kRnD + i] = (float)(acc[j] * norm);
+}
+static_assert(kRnX % kRtJ == 0 && kRnD <= 224, "R table tiling");
+static_assert(kRkernElems * sizeof(double) <= kRquadElems * sizeof(float4), "the kernel table fits rquad's buffer");
 
 __global__ void k_fields(FieldArgs F)
 {
@@ -319,21 +417,30 @@ cudaError_t add_counters_batch(unsigned long long* const* dst, const unsigned lo
     return cudaGetLastError();
 }
 
-size_t line_tables_work_doubles() { return 64 + (size_t)kRnX * (kUsNu - 1); }
+// Scratch of the table builds: coefficients, sampler masses, guide edges, R masses.
+constexpr size_t kWorkMass = 64, kWorkLt = kWorkMass + kUsMasses, kWorkR = kWorkLt + kGuideN;
+size_t line_tables_work_doubles() { return kWorkR + kRMasses; }
 
 cudaError_t build_line_tables(double a, const LineTables& T, bool with_r, cudaStream_t s)
 {
     const int N = kWeidemanN;
     const double L = weideman_L(N);
     double* coef = T.work;
-    k_weideman<<<1, 64, 0, s>>>(coef, N, L);
-    k_voigt<<<(kVoigtN + 255) / 256, 256, 0, s>>>(a, coef, N, L, T.voigt_lnH, T.H0);
-    k_usampler<<<kUsNx, 256, 0, s>>>(a, T.us_x, T.us_lncdf, T.us_guide);
+    double* us_mass = T.work + kWorkMass;
+    double* lt = T.work + kWorkLt;
+    double* p = T.work + kWorkR;
+    const int values = kUsMasses + kGuideN + (with_r ? kRMasses : 0);
+    k_line_stage1<<<N + (values + kCoefBlock - 1) / kCoefBlock, kCoefBlock, 0, s>>>(a, coef, N, L, us_mass, lt,
+                                                                                  with_r ? p : nullptr);
+    k_voigt<<<(kVoigtN + kVoigtBlock - 1) / kVoigtBlock, kVoigtBlock, 0, s>>>(a, coef, N, L, T.voigt_lnH, T.H0);
+    k_usampler<<<kUsNx, 256, 0, s>>>(us_mass, lt, T.us_x, T.us_lncdf, T.us_guide);
     if (with_r) {
-        double* p = T.work + 64;
-        k_rmasses<<<(kRnX + 127) / 128, 128, 0, s>>>(a, p);
-        k_rtable<<<(unsigned)((kRtabElems + 255) / 256), 256, 0, s>>>(p, T.rtab);
-        if (T.rquad) k_rquad<<<(unsigned)((kRquadElems + 255) / 256), 256, 0, s>>>(T.rtab, T.rquad);
+        // the kernel table lives in rquad's buffer until k_rquad fills that
+        double* kern = reinterpret_cast<double*>(T.rquad);
+        k_rkernel<<<dim3(kUsNu - 1, kRnG), 224, 0, s>>>(kern);
+        k_rnorm<<<kRnX, 256, 0, s>>>(p);
+        k_rtable<<<dim3(kRnX / kRtJ, kRnG), 224, 0, s>>>(p, kern, T.rtab);
+        k_rquad<<<(unsigned)((kRquadElems + 255) / 256), 256, 0, s>>>(T.rtab, T.rquad);
     }
     return cudaGetLastError();
 }
@@ -342,7 +449,7 @@ cudaError_t build_voigt2d(float* out, double* work, cudaStream_t s)
 {
     const int N = kWeidemanN;
     const double L = weideman_L(N);
-    k_weideman<<<1, 64, 0, s>>>(work, N, L);
+    k_weideman<<<N, kCoefBlock, 0, s>>>(work, N, L);
     k_voigt2d<<<(kV2Na * kV2Nx + 255) / 256, 256, 0, s>>>(work, N, L, out);
     return cudaGetLastError();
 }
