@@ -56,7 +56,8 @@ constexpr int kSmemUsC = kVoigtN + 48;            // 40 x 251 floats
 constexpr int kSmemFloats = kSmemUsC + kUsNx * kUsNu;
 constexpr int kSmemGuideBytes = kUsNx * kGuideN;  // uint8 after the floats
 constexpr int kSmemRowGuide = kSmemFloats * (int)sizeof(float) + kSmemGuideBytes;   // byte offset
-constexpr size_t kSmemBytes = (size_t)kSmemRowGuide + 192;
+constexpr int kSmemRowBins = (kSmemRowGuide + 192 + 15) / 16 * 16;  // FP32 walk: float4 [2 kRowGuideN], float2 [kUsNx]
+constexpr size_t kSmemBytes = (size_t)kSmemRowBins + 2 * kRowGuideN * 16 + kUsNx * 8;
 
 // ---------------------------------------------------------------- compile-time walk features
 enum : unsigned {
@@ -132,6 +133,7 @@ struct TransportArgs {
     unsigned long long max_iters;
     unsigned max_iters32;     // min(max_iters, 2^32 - 1): the per-event check in 32 bits
     int refill_min;
+    int even_fill;            // no more packets than lanes in the grid: equal shares, no work counter
     // line-profile mode (krl_line_desc.ph_mode: 2, or 1 / 3 below)
     int ph_mode;
     const float* voigt2d;     // [kV2Na][kV2Nx] ln H, mode 1

@@ -232,7 +232,10 @@ __device__ __forceinline__ R voigt(R x, const float* sv, R a, R H0)
     i = i < 0 ? 0 : (i > kVoigtN - 2 ? kVoigtN - 2 : i);
     const R f = t - (R)i;
     const R l0 = (R)sv[i], l1 = (R)sv[i + 1];
-    R h = O::ex(((R)1 - f) * l0 + f * l1);
+    R lh;
+    if constexpr (sizeof(R) == 4) lh = fmaf(f, l1, __fmul_rn(1.0f - f, l0));
+    else lh = ((R)1 - f) * l0 + f * l1;
+    R h = O::ex(lh);
     if (ax < (R)1e-4 || ax > (R)1e3) {
         const R ax2 = ax * ax;
         R wing;
@@ -300,25 +303,77 @@ __device__ __forceinline__ R profile(const TransportArgs& A, R x, const float* s
     else return voigt<R>(x, sv, a, H0);
 }
 
+// The sampling tables as the walk reads them (shared memory in profile mode
+// 2). rb and rx serve the FP32 walk. Per bin of the row guide, two vectors:
+// {node x_i+1, or infinity in the last row; i; x_i, 1 / (x_i+1 - x_i)} and
+// {x_i+1, 1 / (x_i+2 - x_i+1); -, -}. Per row, {x_i, 1 / (x_i+1 - x_i)}.
+struct Tabs {
+    const float* sv;
+    const float* sx;
+    const float* sc;
+    const unsigned char* sg;
+    const unsigned char* rg;
+    const float4* rb;
+    const float2* rx;
+};
+
+__device__ __forceinline__ int row_bin(float f)
+{
+    const int t = (int)(__float_as_uint(f) >> 19) - (int)kRowGuideBase;
+    return t < 0 ? 0 : (t > kRowGuideN - 1 ? kRowGuideN - 1 : t);
+}
+
+// The same bin with the clamp on ax itself, which shortens the way from ax to
+// the address (a group's walk waits for it).
+__device__ __forceinline__ int row_bin_in(float ax)
+{
+    const float f = fminf(fmaxf(ax, 0.25f), 511.0f);
+    return (int)(__float_as_uint(f) >> 19) - (int)kRowGuideBase;
+}
+
 // Largest row i in [0, 38] with X[i] <= ax, and the two bracketing nodes:
 // the row guide's entry for the bin of ax (a node at or below ax), then one
 // step up if the next node is also <= ax. The FP64 walk takes the bin of ax
 // rounded toward zero, so the entry stays at or below ax there too.
-template <typename R>
-__device__ __forceinline__ int us_row2(R ax, const float* sx, const unsigned char* rg, R& x0, R& x1)
+__device__ __forceinline__ int us_row2(double ax, const Tabs& T, double& x0, double& x1)
 {
-    float f;
-    if constexpr (sizeof(R) == 4) f = ax;
-    else f = __double2float_rz(ax);
-    int t = (int)(__float_as_uint(f) >> 19) - (int)kRowGuideBase;
-    t = t < 0 ? 0 : (t > kRowGuideN - 1 ? kRowGuideN - 1 : t);
-    const int i = rg[t];
-    const R g0 = (R)sx[i], g1 = (R)sx[i + 1];
-    const R gp = (R)sx[i < kUsNx - 2 ? i + 2 : kUsNx - 1];
+    const float* sx = T.sx;
+    const int i = T.rg[row_bin(__double2float_rz(ax))];
+    const double g0 = (double)sx[i], g1 = (double)sx[i + 1];
+    const double gp = (double)sx[i < kUsNx - 2 ? i + 2 : kUsNx - 1];
     const bool up = i < kUsNx - 2 && g1 <= ax;
     x0 = up ? g1 : g0;
     x1 = up ? gp : g1;
     return i + (up ? 1 : 0);
+}
+
+// The same row for the FP32 walk: one 8-byte read.
+__device__ __forceinline__ int us_row(float ax, const Tabs& T)
+{
+    const float2 g = *reinterpret_cast<const float2*>(T.rb + 2 * row_bin(ax));
+    return __float_as_int(g.y) + (g.x <= ax ? 1 : 0);
+}
+
+// Weight of row i + 1 at ax (the FP32 walk): (ax - x_i) / (x_i+1 - x_i) as a
+// product with the row's approximate reciprocal, which is what __fdividef
+// evaluates (equal for every ax of every row).
+__device__ __forceinline__ float us_weight(float ax, int i, const Tabs& T)
+{
+    const float2 r = T.rx[i];
+    return __fmul_rn(ax - r.x, r.y);
+}
+
+// The FP32 walk's sums and products that two pieces of code share (a lane's
+// walk and a group's, transport_tail.cuh) are written with explicit fused
+// operations: their rounding then does not depend on what the compiler fuses
+// around them, and a packet takes the same path in both.
+
+// u of the two rows interpolated in |x| (for x >= 0; u is odd in x).
+template <typename R>
+__device__ __forceinline__ R us_lerp(R t, R ua, R ub)
+{
+    if constexpr (sizeof(R) == 4) return fmaf(1.0f - t, ua, __fmul_rn(t, ub));
+    else return ((R)1 - t) * ua + t * ub;
 }
 
 // u_par for incoming gas-frame frequency x (|x| <= 300), given L = ln(xi)
@@ -328,18 +383,24 @@ __device__ __forceinline__ int us_row2(R ax, const float* sx, const unsigned cha
 // linear between nodes j and j + 1; the two rows' u are interpolated in |x|.
 // The two rows are walked together so their shared-memory loads overlap.
 template <typename R>
-__device__ __forceinline__ R us_sample(R x, R L, int m, const float* sx, const float* sc, const unsigned char* sg,
-                                       const unsigned char* rg)
+__device__ __forceinline__ R us_sample(R x, R L, int m, const Tabs& T)
 {
     using O = Ops<R>;
     const R ax = fabs(x);
-    R x0, x1;
-    const int i = us_row2(ax, sx, rg, x0, x1);
-    const R t = O::dv(ax - x0, x1 - x0);
-    const float* ra = sc + i * kUsNu;
+    R t;
+    int i;
+    if constexpr (sizeof(R) == 4) {
+        i = us_row(ax, T);
+        t = us_weight(ax, i, T);
+    } else {
+        R x0, x1;
+        i = us_row2(ax, T, x0, x1);
+        t = O::dv(ax - x0, x1 - x0);
+    }
+    const float* ra = T.sc + i * kUsNu;
     const float* rb = ra + kUsNu;
-    int ja = sg[i * kGuideN + m];
-    int jb = sg[(i + 1) * kGuideN + m];
+    int ja = T.sg[i * kGuideN + m];
+    int jb = T.sg[(i + 1) * kGuideN + m];
     R a0 = (R)ra[ja], a1 = (R)ra[ja + 1];
     R b0 = (R)rb[jb], b1 = (R)rb[jb + 1];
     // Every row starts at the floor ln 1e-30 < L and ends at ln 1 = 0 > L
@@ -374,7 +435,7 @@ __device__ __forceinline__ R us_sample(R x, R L, int m, const float* sx, const f
         ua_ = (R)kUsU0 + (R)kUsDu * (R)ja + (R)kUsDu * O::dv(L - a0, a1 - a0);
         ub_ = (R)kUsU0 + (R)kUsDu * (R)jb + (R)kUsDu * O::dv(L - b0, b1 - b0);
     }
-    const R u = ((R)1 - t) * ua_ + t * ub_;
+    const R u = us_lerp<R>(t, ua_, ub_);
     return x < (R)0 ? -u : u;
 }
 
@@ -391,6 +452,11 @@ __device__ __forceinline__ int us_bin(R xi, R& L)
 }
 
 // ---------------------------------------------------------------- packet state
+
+// Per-lane event counters (summed over the CTA at the end of a model).
+struct LaneStats {
+    unsigned long long emit, esc, des, stuck, scat, cross, absorbed;
+};
 
 template <typename R>
 struct Pkt {
@@ -417,7 +483,8 @@ struct Pkt {
 template <typename R>
 __device__ __forceinline__ R vdot(R nx, R ny, R nz, const float4& rec)
 {
-    return fma(nz, (R)rec.w, fma(ny, (R)rec.z, nx * (R)rec.y));
+    if constexpr (sizeof(R) == 4) return fmaf(nz, rec.w, fmaf(ny, rec.z, __fmul_rn(nx, rec.y)));
+    else return fma(nz, (R)rec.w, fma(ny, (R)rec.z, nx * (R)rec.y));
 }
 
 // The FP64 walk keeps 1 / n with the direction (its face distances are
@@ -744,19 +811,18 @@ __device__ __forceinline__ bool append_segment(const TransportArgs& A, int c, fl
 // and the camera-directed emissivity (Eq. scat-line). With a segment buffer
 // (FP32 walk) the emissivity is deposited by the second stage instead.
 template <typename R, unsigned F>
-__device__ void rich_segment(const TransportArgs& A, const Pkt<R>& p, R ds, R xcom, R H, R w)
+__device__ void rich_segment(const TransportArgs& A, int c, const float4& rec, R nx, R ny, R nz, R ds, R xcom, R H, R w)
 {
     if ((A.rich & KRL_TALLY_J) && A.n_ch > 0) {
         R q = Ops<R>::dv(-xcom - (R)A.ch_x0, (R)A.ch_dx);
-        if (q >= (R)0 && q < (R)A.n_ch) atomicAdd(A.J + (size_t)p.c * A.n_ch + (int)q, (double)(w * ds));
+        if (q >= (R)0 && q < (R)A.n_ch) atomicAdd(A.J + (size_t)c * A.n_ch + (int)q, (double)(w * ds));
     }
     if (!(A.rich & KRL_TALLY_EMISS) || A.n_ch <= 0) return;
-    const R base = w * ds * (R)p.rec.x * H * (R)0.079577471545947668;   // 1 / 4 pi
+    const R base = w * ds * (R)rec.x * H * (R)0.079577471545947668;   // 1 / 4 pi
     if constexpr (sizeof(R) == 4) {
-        if (A.seg && append_segment(A, p.c, base, xcom, p.nx, p.ny, p.nz)) return;
+        if (A.seg && append_segment(A, c, base, xcom, nx, ny, nz)) return;
     }
-    for (int m = 0; m < A.n_cam; ++m)
-        emiss_camera<R, (F & F_VEL) != 0>(A, m, p.c, p.rec, p.nx, p.ny, p.nz, xcom, base);
+    for (int m = 0; m < A.n_cam; ++m) emiss_camera<R, (F & F_VEL) != 0>(A, m, c, rec, nx, ny, nz, xcom, base);
 }
 
 // Second stage of the emissivity deposit. A warp takes 32 consecutive
@@ -818,13 +884,17 @@ __global__ void __launch_bounds__(kDepositBlock) k_emiss_deposit(const __grid_co
     }
 }
 
+// lead: whether this lane writes (false in the other lanes of a group that
+// walks one packet together).
 template <typename R, unsigned F>
-__device__ __forceinline__ void flush_visit(const TransportArgs& A, Pkt<R>& p)
+__device__ __forceinline__ void flush_visit(const TransportArgs& A, Pkt<R>& p, bool lead = true)
 {
     if constexpr (sizeof(R) == 8) p.cellsum += p.vis_scat * (uint32_t)p.c;
-    if ((F & F_SCAT) && p.vis_scat && A.scat) atomicAdd(A.scat + p.c, (unsigned long long)p.vis_scat);
-    if ((F & F_RICH) && (A.rich & KRL_TALLY_EXC) && p.vis_exc != (R)0) atomicAdd(A.exc + p.c, (double)p.vis_exc);
-    if ((F & F_RICH) && A.tau_abs && p.vis_abs != (R)0) atomicAdd(A.absw + p.c, (double)p.vis_abs);
+    if (lead) {
+        if ((F & F_SCAT) && p.vis_scat && A.scat) atomicAdd(A.scat + p.c, (unsigned long long)p.vis_scat);
+        if ((F & F_RICH) && (A.rich & KRL_TALLY_EXC) && p.vis_exc != (R)0) atomicAdd(A.exc + p.c, (double)p.vis_exc);
+        if ((F & F_RICH) && A.tau_abs && p.vis_abs != (R)0) atomicAdd(A.absw + p.c, (double)p.vis_abs);
+    }
     p.vis_scat = 0;
     p.vis_exc = (R)0;
     p.vis_abs = (R)0;
@@ -843,11 +913,6 @@ __device__ __forceinline__ T warp_sum(T v)
 // registers and run 256-thread CTAs.
 template <typename R, unsigned F>
 constexpr int max_block() { return (sizeof(R) == 4 && !(F & F_RICH)) ? 512 : 256; }
-
-// Per-lane event counters (summed over the CTA at the end of a model).
-struct LaneStats {
-    unsigned long long emit, esc, des, stuck, scat, cross, absorbed;
-};
 
 // ---------------------------------------------------------------- tail compaction
 //
@@ -870,8 +935,9 @@ constexpr int kBulkCheck = 16;
 template <typename R, unsigned F>
 constexpr int stash_words() { return 9 + (sizeof(R) == 8 ? 1 : 0) + ((F & F_RICH) ? 9 : 8) * (int)(sizeof(R) / 4); }
 
+// (the stash, or the buffers of the last packets' walk in its place)
 template <typename R, unsigned F>
-constexpr size_t smem_bytes(int block) { return kStashOff + (size_t)stash_words<R, F>() * 4u * (size_t)block; }
+constexpr size_t smem_bytes(int block);
 
 template <typename R>
 __device__ __forceinline__ void put_r(uint32_t* w, int& f, int n, int slot, R v)
@@ -973,21 +1039,123 @@ __device__ __forceinline__ R seg_factor(R dt, R& ab)
     return ab / dt;
 }
 
+// Whether the point q lies inside the unit cell ([0, 1] on every axis; false
+// for a NaN).
+__device__ __forceinline__ bool in_cell(float2 qxy, float qz)
+{
+    const float2 hxy = __fadd2_rn(qxy, make_float2(-0.5f, -0.5f));
+    return fabsf(hxy.x) <= 0.5f && fabsf(hxy.y) <= 0.5f && fabsf(qz - 0.5f) <= 0.5f;
+}
+
+// FP32: distance to the nearest face ahead, the axis and 1/n of that face;
+// the packet is moved there. A zero component counts as +1e-30 (the packet
+// then crosses that face only from exactly on it), so that 1/n is finite and
+// its sign alone selects the face ahead.
+__device__ __forceinline__ float to_face(Pkt<float>& p, int& axis, float& nd)
+{
+    using O = Ops<float>;
+    const float ix = O::rcp(p.nx != 0.0f ? p.nx : 1e-30f);
+    const float iy = O::rcp(p.ny != 0.0f ? p.ny : 1e-30f);
+    const float iz = O::rcp(p.nz != 0.0f ? p.nz : 1e-30f);
+    float s = face_dist<float>(p.px, p.nx, ix);
+    nd = ix;
+    axis = 0;
+    const float ty = face_dist<float>(p.py, p.ny, iy);
+    const float tz = face_dist<float>(p.pz, p.nz, iz);
+    if (ty < s) { s = ty; axis = 1; nd = iy; }
+    if (tz < s) { s = tz; axis = 2; nd = iz; }
+    p.px = O::step01(p.px, s, p.nx);
+    p.py = O::step01(p.py, s, p.ny);
+    p.pz = O::step01(p.pz, s, p.nz);
+    return s;
+}
+
+// A packet's end: status 1 escaped, 2 destroyed, 3 budget, 4 absorbed.
+template <typename R>
+__device__ __forceinline__ void end_packet(const TransportArgs& A, const Pkt<R>& p, uint16_t status,
+                                           unsigned long long& counter, LaneStats& st)
+{
+    ++counter;
+    st.scat += p.nscat;
+    st.cross += p.ncross;
+    write_record(A, p, status);
+}
+
+// The packet, moved to the face on `axis` at distance s, enters the next
+// cell. Returns false if it leaves the domain.
+template <typename R, unsigned F>
+__device__ __forceinline__ bool cross_face(const TransportArgs& A, Pkt<R>& p, R alpha, R s, int axis, R nd,
+                                           LaneStats& st, bool lead = true)
+{
+    if constexpr (sizeof(R) == 4) p.tau = fmaxf(0.0f, fmaf(-alpha, s, p.tau));   // (the two tests may part at a tie)
+    else p.tau -= alpha * s;
+    ++p.ncross;
+    flush_visit<R, F>(A, p, lead);
+    const int dim = axis == 0 ? A.nx : (axis == 1 ? A.ny : A.nz);
+    const int stride = axis == 0 ? 1 : (axis == 1 ? A.nx : A.nx * A.ny);
+    const int cur = axis == 0 ? p.cx : (axis == 1 ? p.cy : p.cz);
+    // side from the sign of 1/n, which selected the face
+    const int step = nd > (R)0 ? 1 : -1;
+    int nc = cur + step;
+    int dc = step * stride;
+    const R pnew = step > 0 ? (R)0 : (R)1;
+    if (axis == 0) p.px = pnew;
+    else if (axis == 1) p.py = pnew;
+    else p.pz = pnew;
+    if (nc < 0 || nc >= dim) {
+        if (!((A.periodic >> axis) & 1u)) {
+            if (lead) {
+                spectrum_add(A, (double)p.x, (double)p.wgt);
+                end_packet(A, p, 1, st.esc, st);
+            }
+            return false;
+        }
+        if (nc < 0) { nc += dim; dc += dim * stride; }
+        else { nc -= dim; dc -= dim * stride; }
+    }
+    if (axis == 0) p.cx = nc;
+    else if (axis == 1) p.cy = nc;
+    else p.cz = nc;
+    p.c += dc;
+    p.rec = __ldg(A.cells + p.c);
+    return true;
+}
+
+// Cosine g of the scattering angle as g - 1, and sin(gamma).
+template <typename R>
+__device__ __forceinline__ void scatter_angle(R nx, R ny, R nz, R mx, R my, R mz, R& gm1, R& sg)
+{
+    R g, s2;
+    if constexpr (sizeof(R) == 4) {
+        g = fmaf(nz, mz, fmaf(nx, mx, __fmul_rn(ny, my)));
+        s2 = fmaf(-g, g, 1.0f);
+    } else {
+        g = nx * mx + ny * my + nz * mz;
+        s2 = (R)1 - g * g;
+    }
+    sg = Ops<R>::sq(fmax((R)0, s2));
+    gm1 = g - (R)1;
+}
+
+// x_out = x_in + u_par (g - 1) + u_perp sin(gamma) (Eq. riia-scatter).
+template <typename R>
+__device__ __forceinline__ R scatter_x(R xcom, R upar, R gm1, R z1, R sg)
+{
+    if constexpr (sizeof(R) == 4) return fmaf(z1, sg, fmaf(upar, gm1, xcom));
+    else return xcom + upar * gm1 + z1 * sg;
+}
+
 // Advances an active packet by one event in its current cell (a scattering
 // inside the cell or a crossing of the nearest face). Returns false when the
 // packet has ended (escape, destruction or event budget).
 template <typename R, unsigned F, int PH>
-__device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys& K, Pkt<R>& p, const float* sv,
-                                        const float* sx, const float* sc, const unsigned char* sg,
-                                        const unsigned char* rg, R a, R H0, LaneStats& st)
+__device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys& K, Pkt<R>& p, const Tabs& T, R a, R H0,
+                                        LaneStats& st)
 {
     using O = Ops<R>;
     if (p.nscat + p.ncross >= A.max_iters32) {
         flush_visit<R, F>(A, p);
-        ++st.stuck;
-        st.scat += p.nscat;
-        st.cross += p.ncross;
-        write_record(A, p, 3);
+        end_packet(A, p, 3, st.stuck, st);
         return false;
     }
     // Draw the next scattering's random numbers up front, for every lane of
@@ -1005,8 +1173,10 @@ __device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys&
     }
     const R vdn = (F & F_VEL) ? vdot<R>(p.nx, p.ny, p.nz, p.rec) : (R)0;
     const R xcom = p.x - vdn;
-    const R H = profile<R, PH>(A, xcom, sv, a, H0);
-    const R alpha = (R)p.rec.x * H;
+    const R H = profile<R, PH>(A, xcom, T.sv, a, H0);
+    R alpha;
+    if constexpr (sizeof(R) == 4) alpha = __fmul_rn(p.rec.x, H);
+    else alpha = (R)p.rec.x * H;
     bool scat;
     R ds, sx_ = (R)0, nd = (R)0;
     int axis = 0;
@@ -1018,29 +1188,14 @@ __device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys&
         ds = O::dv(p.tau, alpha);
         const float2 qxy = __ffma2_rn(make_float2(ds, ds), make_float2(p.nx, p.ny), make_float2(p.px, p.py));
         const float qz = fmaf(ds, p.nz, p.pz);
-        const float2 hxy = __fadd2_rn(qxy, make_float2(-0.5f, -0.5f));
-        scat = fabsf(hxy.x) <= 0.5f && fabsf(hxy.y) <= 0.5f && fabsf(qz - 0.5f) <= 0.5f;
+        scat = in_cell(qxy, qz);
         if (scat) {
             p.px = qxy.x;
             p.py = qxy.y;
             p.pz = qz;
         } else {
-            // a zero component counts as +1e-30 (the packet then crosses that
-            // face only from exactly on it), so that 1/n is finite and its
-            // sign alone selects the face ahead
-            const float ix = O::rcp(p.nx != 0.0f ? p.nx : 1e-30f);
-            const float iy = O::rcp(p.ny != 0.0f ? p.ny : 1e-30f);
-            const float iz = O::rcp(p.nz != 0.0f ? p.nz : 1e-30f);
-            sx_ = face_dist<R>(p.px, p.nx, ix);
-            nd = ix;
-            const R ty = face_dist<R>(p.py, p.ny, iy);
-            const R tz = face_dist<R>(p.pz, p.nz, iz);
-            if (ty < sx_) { sx_ = ty; axis = 1; nd = iy; }
-            if (tz < sx_) { sx_ = tz; axis = 2; nd = iz; }
+            sx_ = to_face(p, axis, nd);
             ds = sx_;
-            p.px = O::step01(p.px, ds, p.nx);
-            p.py = O::step01(p.py, ds, p.ny);
-            p.pz = O::step01(p.pz, ds, p.nz);
         }
     } else {
         // FP64 (the lockstep walk): nearest face first, as the oracle does
@@ -1062,17 +1217,14 @@ __device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys&
         // then decays by the continuum's absorption over it
         R wseg = p.wgt, ab = (R)0;
         if (A.tau_abs) wseg = p.wgt * seg_factor<R>((R)__ldg(A.tau_abs + p.c) * ds, ab);
-        if (A.rich & KRL_TALLY_EXC) p.vis_exc += wseg * ds * H;
-        if (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)) rich_segment<R, F>(A, p, ds, xcom, H, wseg);
+        if (A.rich & KRL_TALLY_EXC) p.vis_exc = fma(wseg * ds, H, p.vis_exc);
+        if (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)) rich_segment<R, F>(A, p.c, p.rec, p.nx, p.ny, p.nz, ds, xcom, H, wseg);
         if (A.tau_abs) {
-            p.vis_abs += p.wgt * ab;
+            p.vis_abs = fma(p.wgt, ab, p.vis_abs);
             p.wgt = p.wgt * ((R)1 - ab);
             if (p.wgt < (R)kWeightCut) {
                 flush_visit<R, F>(A, p);
-                ++st.absorbed;
-                st.scat += p.nscat;
-                st.cross += p.ncross;
-                write_record(A, p, 4);
+                end_packet(A, p, 4, st.absorbed, st);
                 return false;
             }
         }
@@ -1090,10 +1242,7 @@ __device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys&
         if ((F & F_RICH) && (A.rich & kRichEps)) {
             if (O::uni(w1.w[2]) < (R)__ldg(A.eps + p.c)) {
                 flush_visit<R, F>(A, p);
-                ++st.des;
-                st.scat += p.nscat;
-                st.cross += p.ncross;
-                write_record(A, p, 2);
+                end_packet(A, p, 2, st.des, st);
                 return false;
             }
         }
@@ -1124,51 +1273,27 @@ __device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys&
             z1 = rad * bc;
             z2 = rad * bs;
         }
-        const R us = us_sample<R>(xcom, L, gm, sx, sc, sg, rg);   // finite for any x; unused beyond 300
+        const R us = us_sample<R>(xcom, L, gm, T);   // finite for any x; unused beyond 300
         const R upar = fabs(xcom) > (R)300 ? z2 : us;
-        const R g = p.nx * mx + p.ny * my + p.nz * mz;
-        const R sg_ = O::sq(fmax((R)0, (R)1 - g * g));
-        const R xout = xcom + upar * (g - (R)1) + z1 * sg_;
+        R gm1, sg;
+        scatter_angle<R>(p.nx, p.ny, p.nz, mx, my, mz, gm1, sg);
+        const R xout = scatter_x<R>(xcom, upar, gm1, z1, sg);
         set_dir(p, mx, my, mz);
         const R vdo = (F & F_VEL) ? vdot<R>(mx, my, mz, p.rec) : (R)0;
         p.x = xout + vdo;
         p.tau = tau_new;
         return true;
     }
-    // ---- cross the face on `axis`
-    if constexpr (sizeof(R) == 4) p.tau = fmaxf(0.0f, p.tau - alpha * sx_);   // (the two tests may part at a tie)
-    else p.tau -= alpha * sx_;
-    ++p.ncross;
-    flush_visit<R, F>(A, p);
-    const int dim = axis == 0 ? A.nx : (axis == 1 ? A.ny : A.nz);
-    const int stride = axis == 0 ? 1 : (axis == 1 ? A.nx : A.nx * A.ny);
-    const int cur = axis == 0 ? p.cx : (axis == 1 ? p.cy : p.cz);
-    // side from the sign of 1/n, which selected the face
-    const int step = nd > (R)0 ? 1 : -1;
-    int nc = cur + step;
-    int dc = step * stride;
-    const R pnew = step > 0 ? (R)0 : (R)1;
-    if (axis == 0) p.px = pnew;
-    else if (axis == 1) p.py = pnew;
-    else p.pz = pnew;
-    if (nc < 0 || nc >= dim) {
-        if (!((A.periodic >> axis) & 1u)) {
-            spectrum_add(A, (double)p.x, (double)p.wgt);
-            ++st.esc;
-            st.scat += p.nscat;
-            st.cross += p.ncross;
-            write_record(A, p, 1);
-            return false;
-        }
-        if (nc < 0) { nc += dim; dc += dim * stride; }
-        else { nc -= dim; dc -= dim * stride; }
-    }
-    if (axis == 0) p.cx = nc;
-    else if (axis == 1) p.cy = nc;
-    else p.cz = nc;
-    p.c += dc;
-    p.rec = __ldg(A.cells + p.c);
-    return true;
+    return cross_face<R, F>(A, p, alpha, sx_, axis, nd, st);
+}
+
+#include "transport_tail.cuh"
+
+template <typename R, unsigned F>
+constexpr size_t smem_bytes(int block)
+{
+    const size_t stash = (size_t)stash_words<R, F>() * 4u * (size_t)block;
+    return kStashOff + (sizeof(R) == 4 && tail_bytes(block) > stash ? tail_bytes(block) : stash);
 }
 
 // One model's walk by the whole CTA: stage the model's tables in shared
@@ -1208,27 +1333,42 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
     }
     if (threadIdx.x == 0) ctl[0] = 0;
     __syncthreads();
-    const float* sv = sm + kSmemVoigt;
-    const float* sx = PH == 1 ? A.us_x : sm + kSmemUsX;
-    const float* sc = PH == 1 ? A.us_lncdf : sm + kSmemUsC;
+    Tabs T;
+    T.sv = sm + kSmemVoigt;
+    T.sx = PH == 1 ? A.us_x : sm + kSmemUsX;
+    T.sc = PH == 1 ? A.us_lncdf : sm + kSmemUsC;
 #ifdef KRL_TABLES_IN_CONSTANT
     if constexpr (PH == 4) {
-        sv = c_voigt;
-        sx = c_usx;
-        sc = c_uslncdf;
+        T.sv = c_voigt;
+        T.sx = c_usx;
+        T.sc = c_uslncdf;
     }
 #endif
-    const unsigned char* sg = PH == 1 ? A.us_guide : sgw;
+    T.sg = PH == 1 ? A.us_guide : sgw;
     // the sampler's row guide, from the staged nodes (all profile modes)
     unsigned char* rgw = reinterpret_cast<unsigned char*>(sm) + kSmemRowGuide;
+    float4* rbw = reinterpret_cast<float4*>(reinterpret_cast<char*>(sm) + kSmemRowBins);
+    float2* rxw = reinterpret_cast<float2*>(rbw + 2 * kRowGuideN);
+    auto rrow = [&](int i) { return make_float2(T.sx[i], Ops<float>::rcp(T.sx[i + 1] - T.sx[i])); };
     for (int t = threadIdx.x; t < kRowGuideN; t += blockDim.x) {
         const float edge = __uint_as_float((unsigned)(t + (int)kRowGuideBase) << 19);
         int i = 0;
-        while (i < kUsNx - 2 && sx[i + 1] <= edge) ++i;
-        rgw[t] = (unsigned char)i;
+        while (i < kUsNx - 2 && T.sx[i + 1] <= edge) ++i;
+        if constexpr (sizeof(R) == 8) {
+            rgw[t] = (unsigned char)i;
+        } else {
+            const float2 r0 = rrow(i), r1 = i < kUsNx - 2 ? rrow(i + 1) : r0;
+            rbw[2 * t] = make_float4(i < kUsNx - 2 ? T.sx[i + 1] : INFINITY, __int_as_float(i), r0.x, r0.y);
+            rbw[2 * t + 1] = make_float4(r1.x, r1.y, 0.0f, 0.0f);
+        }
+    }
+    if constexpr (sizeof(R) == 4) {
+        for (int i = threadIdx.x; i < kUsNx - 1; i += blockDim.x) rxw[i] = rrow(i);
     }
     __syncthreads();
-    const unsigned char* rg = rgw;
+    T.rg = rgw;
+    T.rb = rbw;
+    T.rx = rxw;
 
     const R a = (R)A.a;
     const R H0 = (R)__ldg(A.H0);
@@ -1260,14 +1400,24 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
             if (lane == 0) stop = *reinterpret_cast<volatile int*>(ctl);
             bool leave = __shfl_sync(kFull, stop, 0) != 0;
             if (!leave && (nidle == 32 || (nidle > 0 && nidle >= A.refill_min))) {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(A.next, (unsigned long long)nidle);
-                base = __shfl_sync(kFull, base, 0);
-                leave = base + (unsigned long long)nidle >= A.n;
-                if (leave && lane == 0) *reinterpret_cast<volatile int*>(ctl) = 1;
+                unsigned long long base = 0, top = A.n;
+                if (A.even_fill) {
+                    // no more packets than lanes: every CTA takes an equal
+                    // share of the ids and every warp an equal share of the
+                    // CTA's, so that the longest packets meet little company
+                    const unsigned long long b0 = A.n * blockIdx.x / gridDim.x, b1 = A.n * (blockIdx.x + 1ull) / gridDim.x;
+                    base = b0 + (b1 - b0) * (unsigned)warp / (unsigned)nwarps;
+                    top = b0 + (b1 - b0) * (unsigned)(warp + 1) / (unsigned)nwarps;
+                    leave = true;
+                } else {
+                    if (lane == 0) base = atomicAdd(A.next, (unsigned long long)nidle);
+                    base = __shfl_sync(kFull, base, 0);
+                    leave = base + (unsigned long long)nidle >= A.n;
+                    if (leave && lane == 0) *reinterpret_cast<volatile int*>(ctl) = 1;
+                }
                 if (!active) {
                     const unsigned long long k = base + __popc(idle & ((1u << lane) - 1u));
-                    if (k < A.n) {
+                    if (k < top) {
                         p.id = A.first + k;
                         ++st.emit;
                         if (emit<R, F>(A, K, p)) {
@@ -1284,20 +1434,44 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
                 bulk = false;
                 __syncthreads();
             }
-        } else if (!bulk && (it == kTailRound || !__any_sync(kFull, active))) {
+        } else if (!bulk && (it >= kTailRound || !__any_sync(kFull, active))) {
             // ---- tail phase, end of a round: count and compact
             const unsigned m = __ballot_sync(kFull, active);
             int* cnt = ctl + 4 + 32 * (round & 1);
-            if (lane == 0) cnt[warp] = __popc(m);
+            const unsigned ms = __ballot_sync(kFull, active && p.nscat >= 2u * p.ncross);
+            if (lane == 0) cnt[warp] = __popc(m) | __popc(ms) << 16;
             __syncthreads();
-            int total = 0, before = 0, busy = 0;
+            int total = 0, before = 0, busy = 0, scatters = 0;
             for (int w = 0; w < nwarps; ++w) {
-                const int c = cnt[w];
+                const int c = cnt[w] & 0xffff;
+                scatters += cnt[w] >> 16;
                 total += c;
                 before += w < warp ? c : 0;
                 busy += c > 0 ? 1 : 0;
             }
             if (total == 0) break;            // CTA-uniform
+            if constexpr (sizeof(R) == 4 && (PH == 2 || PH == 4)) {
+                const int tw = nwarps < kTailWarps ? nwarps : kTailWarps;
+                if (total <= tw * kTailPerWarp && 2 * scatters > total) {     // CTA-uniform
+                    // the last packets, dealt over tw warps: group g of warp
+                    // w walks packet g tw + w
+                    if (active) {
+                        flush_visit<R, F>(A, p);
+                        stash_put<R, F>(stash, n, before + __popc(m & ((1u << lane) - 1u)), p);
+                    }
+                    __syncthreads();
+                    constexpr int G = 32 / kTailPerWarp;
+                    const int q = (int)lane / G * tw + warp;
+                    active = warp < tw && q < total;
+                    if (active) stash_get<R, F>(A, stash, n, q, p);
+                    else if (warp < tw) stash_get<R, F>(A, stash, n, 0, p);      // a state to compute on, not walked
+                    __syncthreads();                  // the buffers take the stash's place
+                    if (warp < tw) {
+                        walk_tail<F, PH>(A, K, p, active, G, reinterpret_cast<TailBuf*>(stash) + warp, T, a, H0, st);
+                    }
+                    break;
+                }
+            }
             if (busy > (total + 31) / 32) {   // CTA-uniform
                 if (active) {
                     flush_visit<R, F>(A, p);
@@ -1313,7 +1487,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
             it = 0;
         }
         if (!bulk) ++it;
-        if (active) active = advance<R, F, PH>(A, K, p, sv, sx, sc, sg, rg, a, H0, st);
+        if (active) active = advance<R, F, PH>(A, K, p, T, a, H0, st);
     }
 
     const unsigned long long tot[7] = {warp_sum(st.emit),  warp_sum(st.esc),  warp_sum(st.des),
