@@ -198,7 +198,8 @@ typedef struct {
                                    256 otherwise (the default there)               */
     int ctas_per_sm;            /* resident CTAs per SM of the persistent grid      */
     int refill_min;             /* a warp takes new packets once at least this many
-                                   of its lanes are idle (1..32)                    */
+                                   of its lanes are idle (1..32); 0: the walk
+                                   chooses from how fast its packets end            */
     uint64_t max_iters;         /* per-packet cap on walk iterations (budget);
                                    0: 2^32 - 1 (the default); larger values are
                                    rejected with KRL_ERR_ARG (the walk counts a

@@ -40,6 +40,7 @@ struct krl_grid {
     float* eps = nullptr;
     float* src_rate = nullptr;
     double* src_cdf = nullptr;
+    int* src_guide = nullptr;
     LineTables tab{};
     // tallies
     double* spec_w = nullptr;
@@ -122,6 +123,7 @@ void free_line(krl_grid* g)
     dfree(g->eps);
     dfree(g->src_rate);
     dfree(g->src_cdf);
+    dfree(g->src_guide);
     dfree(g->tab.voigt_lnH);
     dfree(g->tab.H0);
     dfree(g->tab.us_x);
@@ -247,14 +249,25 @@ void fill_args(const krl_grid* g, TransportArgs& A, uint64_t n, uint64_t first_i
     A.src_profile = L.src_profile;
     A.src_axis = L.src_axis;
     A.band_axis = L.band_axis;
-    for (int k = 0; k < 3; ++k) A.src_pos[k] = L.src_pos[k];
-    A.src_plane = L.src_plane;
+    for (int k = 0; k < 3; ++k) {
+        const double X = L.src_kind == KRL_SRC_POINT ? L.src_pos[k] : L.src_plane;
+        const double f = floor(X);
+        A.src_c[k] = f != f ? 0 : f >= 2147483647.0 ? 2147483647 : (f <= -2147483648.0 ? -2147483647 - 1 : (int)f);
+        A.src_q[k] = X - f;
+        if (X - f == 0.0) A.src_on |= 1u << k;
+    }
     A.band_lo = L.band_lo;
     A.band_hi = L.band_hi;
     A.src_cdf = g->src_cdf;
+    A.src_guide = g->src_guide;
     A.spec_lo = L.spec_xmin;
     A.spec_hi = L.spec_xmax;
     A.spec_n = L.spec_nbins;
+    const double sc = L.spec_nbins / (L.spec_xmax - L.spec_xmin);
+    A.spec_sc = (float)sc;
+    A.spec_off = (float)(-L.spec_xmin * sc);
+    A.spec_msc = (float)(1e-6 * sc);
+    A.spec_moff = (float)(1e-6 * fabs(L.spec_xmin * sc) + 1e-6);
     A.n_ch = L.n_ch;
     A.ch_x0 = L.ch_vmin_cms / g->info.b_cms;
     A.ch_dx = L.ch_dv_cms / g->info.b_cms;
@@ -312,7 +325,7 @@ bool blend_crossing(double a, double* u0)
 
 krl_status resolve_tune(const krl_tune* tune, krl_tune& T)
 {
-    T = krl_tune{KRL_PREC_FP32, 0, 0, 1, 0xFFFFFFFFull, 0, KRL_TABLES_SHARED};
+    T = krl_tune{KRL_PREC_FP32, 0, 0, 0, 0xFFFFFFFFull, 0, KRL_TABLES_SHARED};
     if (tune) {
         if (tune->table_space != KRL_TABLES_SHARED && tune->table_space != KRL_TABLES_CONSTANT)
             return fail(KRL_ERR_ARG, "unknown table_space %d", tune->table_space);
@@ -332,7 +345,7 @@ krl_status resolve_tune(const krl_tune* tune, krl_tune& T)
     }
     if (T.block && (T.block < 32 || T.block > 512 || T.block % 32))
         return fail(KRL_ERR_ARG, "block must be a multiple of 32 in [32, 512]");
-    if (T.refill_min < 1 || T.refill_min > 32) return fail(KRL_ERR_ARG, "refill_min must be in [1, 32]");
+    if (T.refill_min < 0 || T.refill_min > 32) return fail(KRL_ERR_ARG, "refill_min must be in [1, 32]");
     return KRL_OK;
 }
 
@@ -529,6 +542,7 @@ krl_status krl_line_set(krl_grid* g, const krl_line_desc* d, krl_stream st)
     if (e == cudaSuccess && L.src_kind == KRL_SRC_VOLUME) {
         e = dalloc(&g->src_rate, n);
         if (e == cudaSuccess) e = dalloc(&g->src_cdf, n);
+        if (e == cudaSuccess) e = dalloc(&g->src_guide, ((size_t)1 << kCdfGuideBits) + 1);
         g->scan_work_n = emission_cdf_work_doubles(g->ncell);
         if (e == cudaSuccess) e = dalloc(&g->scan_work, g->scan_work_n);
         if (e == cudaSuccess) e = cudaMemcpyAsync(g->src_rate, L.src_rate, n * 4, cudaMemcpyDeviceToDevice, s);
@@ -562,6 +576,7 @@ krl_status krl_line_set(krl_grid* g, const krl_line_desc* d, krl_stream st)
     }
     if (e == cudaSuccess && L.src_kind == KRL_SRC_VOLUME)
         e = emission_cdf(g->src_rate, g->ncell, g->src_cdf, g->scan_work, g->scan_work_n, g->bad, s);
+    if (e == cudaSuccess && L.src_kind == KRL_SRC_VOLUME) e = emission_guide(g->src_cdf, g->ncell, g->src_guide, s);
     if (e != cudaSuccess) {
         free_line(g);
         return cuda_fail(e, "krl_line_set kernels");
@@ -655,6 +670,12 @@ krl_status krl_run_packets(krl_grid* g, uint64_t n, uint64_t first_id, uint64_t 
             A.seg_count = static_cast<unsigned long long*>(segbuf);
             A.seg = reinterpret_cast<float4*>(static_cast<char*>(segbuf) + 16);
             A.seg_cap = cap;
+            // chunks of 256 records while they take at most half the buffer;
+            // below 32 a chunk would not hold a warp's segments
+            const unsigned long long warps = (unsigned long long)grid * (unsigned)(T.block / 32);
+            A.seg_chunk = 256;
+            while (A.seg_chunk >= 32 && A.seg_chunk * warps * 2 > cap) A.seg_chunk >>= 1;
+            if (A.seg_chunk < 32) A.seg_chunk = 0;
         } else {
             (void)cudaGetLastError();
             segbuf = nullptr;

@@ -108,11 +108,18 @@ struct TransportArgs {
     const float* rtab;
     const float4* rquad;      // rtab by interpolation cell (the deposit's second stage)
     int src_kind, src_profile, src_axis, band_axis;
-    double src_pos[3];
-    double src_plane, band_lo, band_hi;
+    // point or plane source: cell, place in the cell and (bit d) whether that
+    // is exactly on its lower face, per fixed axis
+    int src_c[3];
+    unsigned src_on;
+    double src_q[3];
+    double band_lo, band_hi;
     const double* src_cdf;
+    const int* src_guide;     // [2^kCdfGuideBits + 1]: first cell with cdf > bin's lower edge
     double spec_lo, spec_hi;
     int spec_n;
+    float spec_sc, spec_off;  // bin of x: floor(x spec_sc + spec_off), within
+    float spec_msc, spec_moff;    // |x| spec_msc + spec_moff of the FP64 value
     int n_ch;
     double ch_x0, ch_dx;      // v_min / b, dv / b (the FP32 walk rounds them once)
     int n_cam;
@@ -132,7 +139,7 @@ struct TransportArgs {
     RoundKeys keys;           // round keys of (k0, k1)
     unsigned long long max_iters;
     unsigned max_iters32;     // min(max_iters, 2^32 - 1): the per-event check in 32 bits
-    int refill_min;
+    int refill_min;           // 0: the walk chooses
     int even_fill;            // no more packets than lanes in the grid: equal shares, no work counter
     // line-profile mode (krl_line_desc.ph_mode: 2, or 1 / 3 below)
     int ph_mode;
@@ -141,14 +148,20 @@ struct TransportArgs {
     double v2_w;              // mode 1: weight of row v2_row + 1
     double u0;                // mode 3: core-wing crossing point
     // two-stage emissivity deposit (FP32 walk): segment records, 2 float4
-    // each ({cell bits, base, x_com, nx}, {ny, nz, 0, 0}); count may run past
+    // each ({cell bits, base, x_com, nx}, {ny, nz, 0, 0}; cell -1: empty); count may run past
     // the capacity (the segments beyond it are deposited by the walk)
     float4* seg;
     unsigned long long* seg_count;
     unsigned long long seg_cap;
+    unsigned seg_chunk;       // records a warp takes at once (a power of two), or 0
 };
 
 constexpr unsigned kRichEps = 1u << 16;
+
+// Bins of the emission CDF's guide: a search between neighbouring entries
+// takes log2(cells / 65536) steps where a search of the whole CDF takes
+// log2(cells), each a dependent read from L2.
+constexpr int kCdfGuideBits = 16;
 
 // Two-dimensional Voigt table of line-profile mode 1: ln H(a_j, x_i), a_j
 // uniform in log10 a on [kV2LaMin, kV2LaMax], x_i uniform in log10|x| on
@@ -276,6 +289,8 @@ cudaError_t validate_field(const float* f, int n, bool allow_negative, int* bad,
 cudaError_t emission_cdf(const float* rate, int n, double* cdf, double* work, size_t work_doubles,
                          int* bad, cudaStream_t s);
 size_t emission_cdf_work_doubles(int n);
+// guide[b] = first cell with cdf > b 2^-kCdfGuideBits (n - 1 if there is none).
+cudaError_t emission_guide(const double* cdf, int n, int* guide, cudaStream_t s);
 
 // dst[m][k] += src[m * ST_N + k] for m < n_models, k < ST_N (64-bit counters).
 cudaError_t add_counters_batch(unsigned long long* const* dst, const unsigned long long* src, int n_models,

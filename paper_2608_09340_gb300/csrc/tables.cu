@@ -393,6 +393,20 @@ __global__ void k_scan_finish(double* out, int n, const double* offs, int nb)
     out[i] = (out[i] + offs[i / kScanChunk]) / total;
 }
 
+__global__ void k_cdf_guide(const double* cdf, int n, int* guide)
+{
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b > (1 << kCdfGuideBits)) return;
+    const double edge = (double)b / (1 << kCdfGuideBits);
+    int l = 0, h = n - 1;
+    while (l < h) {
+        const int m = (int)(((unsigned)l + (unsigned)h) >> 1);
+        if (cdf[m] > edge) h = m;
+        else l = m + 1;
+    }
+    guide[b] = l;
+}
+
 __global__ void k_add_counters(unsigned long long* out, const unsigned long long* in, int n)
 {
     int i = threadIdx.x;
@@ -478,6 +492,12 @@ cudaError_t emission_cdf(const float* rate, int n, double* cdf, double* work, si
     k_scan_totals<<<1, kScanT, 0, s>>>(work, nb);
     k_scan_total<<<1, 1, 0, s>>>(cdf, n, work, nb, bad);
     k_scan_finish<<<(n + 255) / 256, 256, 0, s>>>(cdf, n, work, nb);
+    return cudaGetLastError();
+}
+
+cudaError_t emission_guide(const double* cdf, int n, int* guide, cudaStream_t s)
+{
+    k_cdf_guide<<<((1 << kCdfGuideBits) + 128) / 128, 128, 0, s>>>(cdf, n, guide);
     return cudaGetLastError();
 }
 

@@ -315,6 +315,7 @@ struct Tabs {
     const unsigned char* rg;
     const float4* rb;
     const float2* rx;
+    unsigned long long* segw;       // this warp's next slot of the segment buffer
 };
 
 __device__ __forceinline__ int row_bin(float f)
@@ -527,16 +528,31 @@ __device__ __forceinline__ void iso_dir(R umu, R uphi, R& nx, R& ny, R& nz)
     nz = mu;
 }
 
-__device__ __forceinline__ void spectrum_add(const TransportArgs& A, double x, double w)
+__device__ __forceinline__ int spectrum_bin(const TransportArgs& A, double x)
 {
-    int b;
-    if (x < A.spec_lo) b = 0;
-    else if (x >= A.spec_hi) b = A.spec_n + 1;
-    else {
-        b = 1 + (int)floor((x - A.spec_lo) / (A.spec_hi - A.spec_lo) * A.spec_n);
-        if (b > A.spec_n) b = A.spec_n;
+    if (x < A.spec_lo) return 0;
+    if (x >= A.spec_hi) return A.spec_n + 1;
+    const int b = 1 + (int)floor((x - A.spec_lo) / (A.spec_hi - A.spec_lo) * A.spec_n);
+    return b > A.spec_n ? A.spec_n : b;
+}
+
+// The FP32 walk finds the bin in single precision and takes the FP64 form
+// (whose divide alone keeps an SM's FP64 pipe busy for some 400 cycles) only
+// where the place in the bin is within the single-precision error of an
+// edge: q = x sc + off has an error below 2e-7 (|x sc| + |off|), the margin
+// is 1e-6 of that sum. Inf and NaN fail both tests.
+template <typename R>
+__device__ __forceinline__ void spectrum_add(const TransportArgs& A, R x, R w)
+{
+    int b = -1;
+    if constexpr (sizeof(R) == 4) {
+        const float q = fmaf(x, A.spec_sc, A.spec_off);
+        const float m = fmaf(fabsf(x), A.spec_msc, A.spec_moff);
+        const float fl = floorf(q), fr = q - fl;
+        if (fr > m && fr < 1.0f - m) b = fl < 0.0f ? 0 : (fl >= (float)A.spec_n ? A.spec_n + 1 : 1 + (int)fl);
     }
-    atomicAdd(A.spec_w + b, w);
+    if (b < 0) b = spectrum_bin(A, (double)x);
+    atomicAdd(A.spec_w + b, (double)w);
     atomicAdd(A.spec_c + b, 1ull);
 }
 
@@ -555,12 +571,50 @@ __device__ __forceinline__ void write_record(const TransportArgs& A, const Pkt<R
     A.rec[p.id - A.first] = r;
 }
 
+// X = dim u, u = (2 (r >> 9) + 1) 2^-24 the uniform of word r: the product is
+// exact in 64-bit integers. Its cell and the place in the cell, as floor(X)
+// and X - floor(X) give them.
+template <typename R>
+__device__ __forceinline__ void place_uniform(int dim, uint32_t r, int& c, R& q, bool& on)
+{
+    const unsigned long long v = (unsigned long long)(unsigned)dim * (2u * (r >> 9) + 1u);
+    const unsigned low = (unsigned)v & 0xffffffu;
+    c = (int)(v >> 24);
+    q = (R)low * (R)0x1p-24;
+    on = low == 0u;
+}
+
+// First cell with cdf > uc, uc = (2 K + 1) 2^-49 with K the 48 bits of two
+// words. The guide's bin (the top 16 bits of uc) bounds it between two
+// neighbouring entries; CDF values are not negative, so their order is that
+// of their bits as integers. Uses no FP64 instruction.
+__device__ __forceinline__ int pick_cell(const TransportArgs& A, uint32_t w0, uint32_t w1)
+{
+    const unsigned long long v = ((unsigned long long)(w0 >> 8) << 25) | (2u * (w1 >> 8) + 1u);
+    const int top = 63 - __clzll((long long)v);                  // uc = 1.x 2^(top - 49)
+    const unsigned long long uc =
+        ((unsigned long long)(1023 + top - 49) << 52) | ((v << (52 - top)) & 0xfffffffffffffull);
+    const unsigned bin = w0 >> (32 - kCdfGuideBits);
+    int l = __ldg(A.src_guide + bin), h = __ldg(A.src_guide + bin + 1);
+    const long long* cdf = reinterpret_cast<const long long*>(A.src_cdf);
+    while (l < h) {
+        const int m = (int)(((unsigned)l + (unsigned)h) >> 1);
+        if (__ldg(cdf + m) > (long long)uc) h = m;
+        else l = m + 1;
+    }
+    return l;
+}
+
 // Emission (event 0). Slots: block 0 = {mu, phi, tau, freq1},
 // block 1 = {freq2, pos_a, pos_b, pos_c}, block 2 = {cell_hi, cell_lo}.
 // Returns false if the source point lies outside the domain (the packet
-// then leaves at once).
+// then leaves at once). The position is formed without FP64 arithmetic
+// (except a beam's band): a warp emits for the few lanes that are idle, and
+// where packets have tens of events the FP64 pipe, at 16 cycles per warp
+// instruction, was the bound of the whole walk (70 % busy on the 128^3
+// cloud, 86 events per packet).
 template <typename R, unsigned F>
-__device__ bool emit(const TransportArgs& A, const RoundKeys& K, Pkt<R>& p)
+__device__ __forceinline__ bool emit(const TransportArgs& A, const RoundKeys& K, Pkt<R>& p)
 {
     using O = Ops<R>;
     const uint32_t lo = (uint32_t)p.id, hi = (uint32_t)(p.id >> 32);
@@ -569,64 +623,72 @@ __device__ bool emit(const TransportArgs& A, const RoundKeys& K, Pkt<R>& p)
     Words b1 = {{0u, 0u, 0u, 0u}};
     if (need1) b1 = philox(lo, hi, 0u, 1u, K);
     const int dims[3] = {A.nx, A.ny, A.nz};
-    double X[3];
-    R n[3];
-    if (A.src_kind == KRL_SRC_BEAM) {
-        n[0] = n[1] = n[2] = (R)0;
-        n[A.src_axis] = (R)1;
-        double pos[2] = {(double)O::uni(b1.w[1]), (double)O::uni(b1.w[2])};
-        int q = 0;
+    R n[3], pp[3];
+    int ci[3];
+    bool on[3];                 // exactly on the cell's lower face
+    if (A.src_kind == KRL_SRC_VOLUME) {
+        iso_dir<R>(O::uni(b0.w[0]), O::uni(b0.w[1]), n[0], n[1], n[2]);
+        const Words b2 = philox(lo, hi, 0u, 2u, K);
+        const int l = pick_cell(A, b2.w[0], b2.w[1]);
+        const int row = l / A.nx;
+        ci[0] = l - row * A.nx;
+        ci[2] = row / A.ny;
+        ci[1] = row - ci[2] * A.ny;
+#pragma unroll
         for (int d = 0; d < 3; ++d) {
-            if (d == A.src_axis) { X[d] = 0.0; continue; }
-            X[d] = (d == A.band_axis) ? A.band_lo + (A.band_hi - A.band_lo) * pos[q] : dims[d] * pos[q];
-            ++q;
+            pp[d] = O::uni(b1.w[1 + d]);
+            on[d] = false;
+        }
+    } else if (A.src_kind == KRL_SRC_BEAM) {
+        int q = 0;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const bool along = d == A.src_axis;
+            n[d] = along ? (R)1 : (R)0;
+            ci[d] = 0;
+            pp[d] = (R)0;
+            on[d] = along;
+            if (!along) {
+                const uint32_t r = q == 0 ? b1.w[1] : b1.w[2];
+                if (d == A.band_axis) {
+                    const double X = A.band_lo + (A.band_hi - A.band_lo) * (double)O::uni(r);
+                    const double f = floor(X);
+                    ci[d] = (int)f;
+                    pp[d] = (R)(X - f);
+                    on[d] = X - f == 0.0;
+                } else {
+                    place_uniform<R>(dims[d], r, ci[d], pp[d], on[d]);
+                }
+                ++q;
+            }
         }
     } else {
         iso_dir<R>(O::uni(b0.w[0]), O::uni(b0.w[1]), n[0], n[1], n[2]);
-        if (A.src_kind == KRL_SRC_POINT) {
-            X[0] = A.src_pos[0];
-            X[1] = A.src_pos[1];
-            X[2] = A.src_pos[2];
-        } else if (A.src_kind == KRL_SRC_PLANE) {
-            int q = 1;
-            for (int d = 0; d < 3; ++d)
-                X[d] = (d == A.src_axis) ? A.src_plane : dims[d] * (double)O::uni(b1.w[q++]);
-        } else {
-            Words b2 = philox(lo, hi, 0u, 2u, K);
-            double uc = (double)(b2.w[0] >> 8) * 0x1p-24 + (double)(b2.w[1] >> 8) * 0x1p-48 + 0x1p-49;
-            int l = 0, h = A.ncell - 1;              // first cell with cdf > uc
-            while (l < h) {
-                int m = (l + h) >> 1;
-                if (A.src_cdf[m] > uc) h = m;
-                else l = m + 1;
-            }
-            int cz = l / (A.nx * A.ny);
-            int cy = (l / A.nx) % A.ny;
-            int cx = l % A.nx;
-            X[0] = cx + (double)O::uni(b1.w[1]);
-            X[1] = cy + (double)O::uni(b1.w[2]);
-            X[2] = cz + (double)O::uni(b1.w[3]);
+        int q = 0;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            ci[d] = A.src_c[d];
+            pp[d] = (R)A.src_q[d];
+            on[d] = (A.src_on >> d) & 1u;
+            if (A.src_kind == KRL_SRC_PLANE && d != A.src_axis)
+                place_uniform<R>(dims[d], q++ == 0 ? b1.w[1] : b1.w[2], ci[d], pp[d], on[d]);
         }
     }
     set_dir(p, n[0], n[1], n[2]);
-    int ci[3];
-    R pp[3];
     bool inside = true;
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-        double f = floor(X[d]);
-        int c = (int)f;
-        double q = X[d] - f;
-        if (q == 0.0 && n[d] < (R)0) {
+        int c = ci[d];
+        if (on[d] && n[d] < (R)0) {
             c -= 1;
-            q = 1.0;
+            pp[d] = (R)1;
         }
-        if ((A.periodic >> d) & 1u) {
+        if (((A.periodic >> d) & 1u) && (c < 0 || c >= dims[d])) {
             c %= dims[d];
             if (c < 0) c += dims[d];
         }
         if (c < 0 || c >= dims[d]) inside = false;
         ci[d] = c;
-        pp[d] = (R)q;
     }
     p.tau = fmax((R)0, -O::ln(O::uni(b0.w[2])));
     R xcom = (R)0;
@@ -786,19 +848,53 @@ __device__ __forceinline__ void emiss_camera(const TransportArgs& A, int m, int 
     for (int k = S.k0; k <= S.k1; ++k, kf += (R)1) emiss_channel<R, false>(A, out, S, xcom, base, k, kf);
 }
 
+// Marks segment records [i, i + n) as empty.
+__device__ __forceinline__ void clear_segments(const TransportArgs& A, unsigned long long i, unsigned n)
+{
+    for (unsigned k = 0; k < n; ++k)
+        if (i + k < A.seg_cap) A.seg[2 * (i + k)] = make_float4(__int_as_float(-1), 0.0f, 0.0f, 0.0f);
+}
+
 // First stage of the two-stage emissivity deposit (FP32 walk): the segment
-// (cell, base weight, x_com, direction) goes to the run's segment buffer,
-// one slot range per converged group of lanes (one atomic on the buffer's
-// counter). Returns false when the buffer is full; the caller then deposits
-// the segment itself.
-__device__ __forceinline__ bool append_segment(const TransportArgs& A, int c, float base, float xcom, float nx,
-                                               float ny, float nz)
+// (cell, base weight, x_com, direction) goes to the run's segment buffer, one
+// slot range per converged group of lanes. A warp takes slots from a chunk of
+// seg_chunk records of its own (*word: the next one; at a multiple of the
+// chunk there is none), so that the buffer's counter takes one atomic per
+// chunk: one per group made that single address the bound of the walk (0.8e6
+// atomics, each waited for, in a 3 ms run). What a chunk has left when a
+// group does not fit is marked empty. seg_chunk 0 (a buffer too small to
+// leave each warp a chunk): every group takes its slots from the counter.
+// Returns false when the buffer is full; the caller then deposits the segment
+// itself.
+__device__ __forceinline__ bool append_segment(const TransportArgs& A, unsigned long long* word, int c, float base,
+                                               float xcom, float nx, float ny, float nz)
 {
     const unsigned mask = __activemask();
     const unsigned lane = threadIdx.x & 31u;
     const int leader = __ffs(mask) - 1;
     unsigned long long first = 0;
-    if ((int)lane == leader) first = atomicAdd(A.seg_count, (unsigned long long)__popc(mask));
+    if ((int)lane == leader) {
+        const unsigned cnt = (unsigned)__popc(mask), chunk = A.seg_chunk;
+        if (chunk == 0u) {
+            first = atomicAdd(A.seg_count, (unsigned long long)cnt);
+        } else {
+            // another group of this warp may take slots in between: the swap
+            // then fails and the new word is looked at (at most 31 times)
+            unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(word);
+            for (;;) {
+                const unsigned left = (unsigned)(0ull - old) & (chunk - 1u);
+                const bool fits = cnt <= left;
+                first = fits ? old : atomicAdd(A.seg_count, (unsigned long long)chunk);
+                const unsigned long long seen = atomicCAS(word, old, first + cnt);
+                if (seen == old) {
+                    if (!fits) clear_segments(A, old, left);
+                    break;
+                }
+                if (!fits) clear_segments(A, first, chunk);
+                old = seen;
+            }
+        }
+    }
     first = __shfl_sync(mask, first, leader);
     const unsigned long long i = first + __popc(mask & ((1u << lane) - 1u));
     if (i >= A.seg_cap) return false;
@@ -811,7 +907,7 @@ __device__ __forceinline__ bool append_segment(const TransportArgs& A, int c, fl
 // and the camera-directed emissivity (Eq. scat-line). With a segment buffer
 // (FP32 walk) the emissivity is deposited by the second stage instead.
 template <typename R, unsigned F>
-__device__ void rich_segment(const TransportArgs& A, int c, const float4& rec, R nx, R ny, R nz, R ds, R xcom, R H, R w)
+__device__ void rich_segment(const TransportArgs& A, const Tabs& T, int c, const float4& rec, R nx, R ny, R nz, R ds, R xcom, R H, R w)
 {
     if ((A.rich & KRL_TALLY_J) && A.n_ch > 0) {
         R q = Ops<R>::dv(-xcom - (R)A.ch_x0, (R)A.ch_dx);
@@ -820,7 +916,7 @@ __device__ void rich_segment(const TransportArgs& A, int c, const float4& rec, R
     if (!(A.rich & KRL_TALLY_EMISS) || A.n_ch <= 0) return;
     const R base = w * ds * (R)rec.x * H * (R)0.079577471545947668;   // 1 / 4 pi
     if constexpr (sizeof(R) == 4) {
-        if (A.seg && append_segment(A, c, base, xcom, nx, ny, nz)) return;
+        if (A.seg && append_segment(A, T.segw, c, base, xcom, nx, ny, nz)) return;
     }
     for (int m = 0; m < A.n_cam; ++m) emiss_camera<R, (F & F_VEL) != 0>(A, m, c, rec, nx, ny, nz, xcom, base);
 }
@@ -845,12 +941,12 @@ __global__ void __launch_bounds__(kDepositBlock) k_emiss_deposit(const __grid_co
     for (unsigned long long w = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) & ~31ull; w < n;
          w += stride) {
         const unsigned long long i = w + (unsigned long long)lane;
-        const bool valid = i < n;
-        float4 r0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), r1 = r0;
-        if (valid) {
+        float4 r0 = make_float4(__int_as_float(-1), 0.0f, 0.0f, 0.0f), r1 = r0;
+        if (i < n) {
             r0 = __ldg(A.seg + 2 * i);
             r1 = __ldg(A.seg + 2 * i + 1);
         }
+        const bool valid = __float_as_int(r0.x) >= 0;       // (not an empty record)
         const int c = valid ? __float_as_int(r0.x) : 0;
         const float4 rec = (VEL && valid) ? __ldg(A.cells + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         const float base = r0.y, xcom = r0.z;
@@ -921,7 +1017,7 @@ constexpr int max_block() { return (sizeof(R) == 4 && !(F & F_RICH)) ? 512 : 256
 // stash that holds one packet per thread, field-major (one 32-bit word per
 // field and slot, so consecutive slots fall in consecutive banks).
 constexpr size_t kCtlOff = (kSmemBytes + 15) / 16 * 16;
-constexpr int kCtlInts = 4 + 2 * 32;
+constexpr int kCtlInts = 4 + 2 * 32 + 2 * 16;         // ... and a 64-bit word per warp
 constexpr size_t kStashOff = kCtlOff + (size_t)kCtlInts * sizeof(int);
 // Events a lane runs between two compaction checks in the tail.
 constexpr int kTailRound = 32;
@@ -1105,7 +1201,7 @@ __device__ __forceinline__ bool cross_face(const TransportArgs& A, Pkt<R>& p, R 
     if (nc < 0 || nc >= dim) {
         if (!((A.periodic >> axis) & 1u)) {
             if (lead) {
-                spectrum_add(A, (double)p.x, (double)p.wgt);
+                spectrum_add(A, p.x, p.wgt);
                 end_packet(A, p, 1, st.esc, st);
             }
             return false;
@@ -1218,7 +1314,7 @@ __device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys&
         R wseg = p.wgt, ab = (R)0;
         if (A.tau_abs) wseg = p.wgt * seg_factor<R>((R)__ldg(A.tau_abs + p.c) * ds, ab);
         if (A.rich & KRL_TALLY_EXC) p.vis_exc = fma(wseg * ds, H, p.vis_exc);
-        if (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)) rich_segment<R, F>(A, p.c, p.rec, p.nx, p.ny, p.nz, ds, xcom, H, wseg);
+        if (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)) rich_segment<R, F>(A, T, p.c, p.rec, p.nx, p.ny, p.nz, ds, xcom, H, wseg);
         if (A.tau_abs) {
             p.vis_abs = fma(p.wgt, ab, p.vis_abs);
             p.wgt = p.wgt * ((R)1 - ab);
@@ -1332,6 +1428,8 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
         for (int i = threadIdx.x; i < kUsNx * kGuideN; i += blockDim.x) sgw[i] = A.us_guide[i];
     }
     if (threadIdx.x == 0) ctl[0] = 0;
+    unsigned long long* segw = reinterpret_cast<unsigned long long*>(ctl + 4 + 2 * 32) + (threadIdx.x >> 5);
+    if ((threadIdx.x & 31u) == 0u) *segw = 0ull;
     __syncthreads();
     Tabs T;
     T.sv = sm + kSmemVoigt;
@@ -1369,6 +1467,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
     T.rg = rgw;
     T.rb = rbw;
     T.rx = rxw;
+    T.segw = segw;
 
     const R a = (R)A.a;
     const R H0 = (R)__ldg(A.H0);
@@ -1383,11 +1482,13 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
     const int n = (int)blockDim.x;
     bool bulk = true;
     int round = 0, it = 0, quiet = 0;
+    int refill = 1, taken = 0, iters = 0;   // idle lanes to wait for; ids taken; bulk iterations
     for (;;) {
         // ---- bulk phase: refill idle lanes, leave when the ids run out. A
         // warp whose lanes are all busy skips this bookkeeping, except every
         // kBulkCheck-th iteration, when it looks at the CTA's stop flag (the
         // other warps may be waiting for it at the tail barrier).
+        ++iters;
         const unsigned idle = bulk ? __ballot_sync(kFull, !active) : 0u;
         if (bulk && (idle != 0u || ++quiet == kBulkCheck)) {
             quiet = 0;
@@ -1399,7 +1500,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
             int stop = 0;
             if (lane == 0) stop = *reinterpret_cast<volatile int*>(ctl);
             bool leave = __shfl_sync(kFull, stop, 0) != 0;
-            if (!leave && (nidle == 32 || (nidle > 0 && nidle >= A.refill_min))) {
+            if (!leave && (nidle == 32 || (nidle > 0 && nidle >= (A.refill_min > 0 ? A.refill_min : refill)))) {
                 unsigned long long base = 0, top = A.n;
                 if (A.even_fill) {
                     // no more packets than lanes: every CTA takes an equal
@@ -1415,6 +1516,16 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
                     leave = base + (unsigned long long)nidle >= A.n;
                     if (leave && lane == 0) *reinterpret_cast<volatile int*>(ctl) = 1;
                 }
+                // The emission runs for the idle lanes alone and costs about as
+                // much as four events of the whole warp: with lambda lanes
+                // ending per iteration, waiting for m idle lanes costs m / 2
+                // lanes and saves all but 1 / m of the emissions' time, best
+                // near m = sqrt(64 x 4 lambda). 1 for long walks.
+                taken += nidle;
+                if (iters >= 32) {
+                    const int m = (int)sqrtf(256.0f * (float)(taken - 32) / (float)iters);
+                    refill = m < 1 ? 1 : (m > 16 ? 16 : m);
+                }
                 if (!active) {
                     const unsigned long long k = base + __popc(idle & ((1u << lane) - 1u));
                     if (k < top) {
@@ -1423,7 +1534,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
                         if (emit<R, F>(A, K, p)) {
                             active = true;
                         } else {
-                            spectrum_add(A, (double)p.x, 1.0);
+                            spectrum_add(A, p.x, (R)1);
                             ++st.esc;
                             write_record(A, p, 1);
                         }
@@ -1490,6 +1601,15 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
         if (active) active = advance<R, F, PH>(A, K, p, T, a, H0, st);
     }
 
+    if constexpr (sizeof(R) == 4 && (F & F_RICH) != 0) {
+        // the rest of the warp's last chunk of segment records
+        if (A.seg && A.seg_chunk) {
+            __syncwarp();
+            const unsigned long long i = *segw;
+            const unsigned left = (unsigned)(0ull - i) & (A.seg_chunk - 1u);
+            for (unsigned k = lane; k < left; k += 32u) clear_segments(A, i + k, 1u);
+        }
+    }
     const unsigned long long tot[7] = {warp_sum(st.emit),  warp_sum(st.esc),  warp_sum(st.des),
                                        warp_sum(st.stuck), warp_sum(st.scat), warp_sum(st.cross),
                                        warp_sum(st.absorbed)};

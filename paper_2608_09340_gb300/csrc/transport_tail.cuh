@@ -416,7 +416,7 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
             (pos < f || (pos == f && ends && scat))) {
             float wseg = ow;
             if (absorbs) wseg = ow * fct;
-            rich_segment<float, F>(A, p.c, p.rec, ix, iy, iz, ds, myc, H, wseg);
+            rich_segment<float, F>(A, T, p.c, p.rec, ix, iy, iz, ds, myc, H, wseg);
         }
         // ---- the state in front of segment f, or after the whole chain
         const bool whole = f == now;
@@ -461,7 +461,7 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
                 if (absorbs) wseg = p.wgt * seg_factor<float>(__ldg(A.tau_abs + p.c) * s, fab);
                 if (A.rich & KRL_TALLY_EXC) p.vis_exc = fmaf(wseg * s, fH, p.vis_exc);
                 if (fk == 1 && lead && (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)))
-                    rich_segment<float, F>(A, p.c, rec, p.nx, p.ny, p.nz, s, fc, fH, wseg);
+                    rich_segment<float, F>(A, T, p.c, rec, p.nx, p.ny, p.nz, s, fc, fH, wseg);
                 if (absorbs) {
                     p.vis_abs = fmaf(p.wgt, fab, p.vis_abs);
                     p.wgt = p.wgt * (1.0f - fab);
