@@ -413,9 +413,9 @@ typedef struct {
     const float* emiss;     /* device [ncell][n_ch] camera-directed scattering
                                emissivity (raw KRL_OUT_EMISS units), or NULL for
                                this grid's tally of `camera`; 4-byte aligned.
-                               When 16-byte aligned and n_ch is 4, 8, 16, 32,
-                               64 or 128, each cell's row is read as 16-byte
-                               vectors (faster; the same result)              */
+                               When 32-byte aligned and n_ch a multiple of 8
+                               (16-byte, of 4), rows are read as 32-byte
+                               (16-byte) vectors (faster; the same result)              */
     const float* jline;     /* device [ncell] frequency-integrated line emission
                                per unit path (same units), or NULL              */
     int no_scratch;         /* nonzero: allocate nothing; evaluate the profile

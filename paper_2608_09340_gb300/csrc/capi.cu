@@ -762,6 +762,8 @@ krl_status krl_raytrace_channels(krl_grid* g, const krl_raytrace_desc* d, float*
     // d < 0, as one FMA; an axis the ray runs parallel to (or whose inverse
     // overflows) gets a distance of 3e38, never the nearest
     for (int k = 0; k < 3; ++k) {
+        A.nh[k] = (float)A.n[k];
+        A.nl[k] = (float)(A.n[k] - (double)A.nh[k]);
         const float d = (float)(-A.n[k]);
         const float inv = 1.0f / d;
         A.dirf[k] = d;

@@ -219,6 +219,7 @@ struct RayArgs {
     int n_ch;
     double ch_x0, ch_dx;      // v_min / b, dv / b
     double n[3], u[3], v[3];  // camera direction and image axes
+    float nh[3], nl[3];       // n as float pairs nh + nl
     float dirf[3];            // the march direction -n in float
     float face_neg[3], face_c[3];   // distance to the face ahead on axis d from in-cell
                                     // position p: fma(p, face_neg[d], face_c[d])

@@ -40,25 +40,45 @@ namespace {
 constexpr int kRtEmin = -16;
 constexpr int kRtEn = 30;
 
-__device__ __forceinline__ float voigt_rt(float x, const float* sv, const int* eI, const float* eF, float a,
-                                          float H0)
+// The tables in shared memory: the slice's neighbouring nodes in pairs and,
+// per exponent, {FT_e, IT_e as bits}: one read each.
+struct ProfileTables {
+    float2 sv[kVoigtN - 1];
+    float2 e[kRtEn];
+};
+
+__device__ __forceinline__ void load_tables(ProfileTables& P, const float* lnH)
+{
+    for (int i = threadIdx.x; i < kVoigtN - 1; i += blockDim.x) P.sv[i] = make_float2(lnH[i], lnH[i + 1]);
+    if (threadIdx.x < kRtEn) {
+        const double t = (double)((kVoigtN - 1) / (kVoigtL1 - kVoigtL0)) *
+                         (((int)threadIdx.x + kRtEmin) * 0.30102999566398119521 - kVoigtL0);
+        const double it = floor(t);
+        P.e[threadIdx.x] = make_float2((float)(t - it), __int_as_float((int)it));
+    }
+}
+
+__device__ __forceinline__ float voigt_rt(float x, const ProfileTables& P, float a, float H0)
 {
     float ax = fabsf(x);
     if (ax < 1e-4f) return H0;
     if (ax > 1e3f) return a / (1.7724538509055160f * ax * ax) * (1.0f + 1.5f / (ax * ax));
-    int e;
-    float m = frexpf(ax, &e);                       // ax = m 2^e, m in [0.5, 1)
-    int q = e - kRtEmin;
+    // ax = m 2^e, m in [0.5, 1): ax is a normal number here, so from its bits
+    const unsigned bits = __float_as_uint(ax);
+    const float m = __uint_as_float((bits & 0x007fffffu) | 0x3f000000u);
+    int q = (int)(bits >> 23) - 126 - kRtEmin;
     q = q < 0 ? 0 : (q > kRtEn - 1 ? kRtEn - 1 : q);
+    const float2 te = P.e[q];
     // C log10(m) = (C log10 2) log2(m); |log2 m| <= 1, so the fast log2's
     // absolute error (~2^-22) moves t by < 5e-5
-    const float sfr = eF[q] + (float)((kVoigtN - 1) / (kVoigtL1 - kVoigtL0) * 0.30102999566398119521) * __log2f(m);
+    const float sfr = te.x + (float)((kVoigtN - 1) / (kVoigtL1 - kVoigtL0) * 0.30102999566398119521) * __log2f(m);
     const float fl = floorf(sfr);
-    int i = eI[q] + (int)fl;
+    int i = __float_as_int(te.y) + (int)fl;
     float f = sfr - fl;
     if (i < 0) { i = 0; f = 0.0f; }
     if (i > kVoigtN - 2) { i = kVoigtN - 2; f = 1.0f; }
-    return __expf((1.0f - f) * sv[i] + f * sv[i + 1]);
+    const float2 v = P.sv[i];
+    return __expf((1.0f - f) * v.x + f * v.y);
 }
 
 // (1 - e^{-d}) / d: from e^{-d} above d = 0.05 (cancellation below 1.2e-6),
@@ -116,25 +136,12 @@ __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v)
 template <int CPL, bool ALPHA>
 __global__ void __launch_bounds__(256) k_rt_profile(const RayArgs A, float* hc)
 {
-    __shared__ float sv[kVoigtN];
-    __shared__ int eI[kRtEn];
-    __shared__ float eF[kRtEn];
-    for (int i = threadIdx.x; i < kVoigtN; i += blockDim.x) sv[i] = A.voigt_lnH[i];
-    if (threadIdx.x < kRtEn) {
-        const double t = (double)((kVoigtN - 1) / (kVoigtL1 - kVoigtL0)) *
-                         (((int)threadIdx.x + kRtEmin) * 0.30102999566398119521 - kVoigtL0);
-        const double it = floor(t);
-        eI[threadIdx.x] = (int)it;
-        eF[threadIdx.x] = (float)(t - it);
-    }
+    __shared__ ProfileTables tabs;
+    load_tables(tabs, A.voigt_lnH);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const long long ncell = (long long)A.nx * A.ny * A.nz;
-    float nh[3], nl[3];
-    for (int d = 0; d < 3; ++d) {
-        nh[d] = (float)A.n[d];
-        nl[d] = (float)(A.n[d] - (double)nh[d]);
-    }
+    const float nh[3] = {A.nh[0], A.nh[1], A.nh[2]}, nl[3] = {A.nl[0], A.nl[1], A.nl[2]};
     float xbh[CPL], xbl[CPL];
 #pragma unroll
     for (int q = 0; q < CPL; ++q) {
@@ -169,9 +176,64 @@ __global__ void __launch_bounds__(256) k_rt_profile(const RayArgs A, float* hc)
                 const int k = lane + 32 * q;
                 if (k < A.n_ch) {
                     const float xk = (xbh[q] - h) + (xbl[q] - l);
-                    const float H = voigt_rt(xk, sv, eI, eF, a, H0);
+                    const float H = voigt_rt(xk, tabs, a, H0);
                     row[k] = ALPHA ? fmaf(ca, H, ct) : H;
                 }
+            }
+        }
+    }
+}
+
+// The same cube when the channels do not fill the lanes (n_ch not a multiple
+// of 32): a warp's 32 cells x n_ch values, which are contiguous, go over its
+// lanes 32 at a time, each lane with the n.V of its value's cell (shuffled)
+// and its channel's frequency (from shared memory). With 5 channels the
+// channel-per-lane form leaves 27 lanes idle.
+template <bool ALPHA>
+__global__ void __launch_bounds__(256) k_rt_profile_flat(const RayArgs A, float* hc)
+{
+    __shared__ ProfileTables tabs;
+    __shared__ float2 xb[128];
+    load_tables(tabs, A.voigt_lnH);
+    for (int k = threadIdx.x; k < A.n_ch; k += blockDim.x) {
+        const double x = -(A.ch_x0 + ((double)k + 0.5) * A.ch_dx);
+        const float h = (float)x;
+        xb[k] = make_float2(h, (float)(x - (double)h));
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const long long ncell = (long long)A.nx * A.ny * A.nz;
+    const float nh[3] = {A.nh[0], A.nh[1], A.nh[2]}, nl[3] = {A.nl[0], A.nl[1], A.nl[2]};
+    const float a = A.a;
+    const float H0 = __ldg(A.H0);
+    const int nch = A.n_ch, dcell = 32 / nch, dk = 32 - dcell * nch;     // 32 values on: cells and channels
+    const long long ngroups = (ncell + 31) / 32;
+    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long grp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; grp < ngroups; grp += nwarps) {
+        const long long c0 = grp * 32;
+        const long long cl = c0 + lane;
+        float vnh = 0.0f, vnl = 0.0f, a0 = 0.0f, ta = 0.0f;
+        if (cl < ncell) {
+            const float4 rec = __ldg(A.cells + cl);
+            a0 = rec.x;
+            if (ALPHA && A.tau_abs) ta = __ldg(A.tau_abs + cl);
+            dot_ff(nh, nl, rec.y, rec.z, rec.w, vnh, vnl);
+        }
+        const int values = (ncell - c0 < 32 ? (int)(ncell - c0) : 32) * nch;
+        float* out = hc + (size_t)c0 * nch;
+        int cell = lane / nch, k = lane - cell * nch;
+        for (int e0 = 0; e0 < values; e0 += 32) {
+            // (past the last value the cell index is masked: not stored)
+            const float h = __shfl_sync(0xffffffffu, vnh, cell & 31), l = __shfl_sync(0xffffffffu, vnl, cell & 31);
+            const float ca = __shfl_sync(0xffffffffu, a0, cell & 31), ct = __shfl_sync(0xffffffffu, ta, cell & 31);
+            const float2 x = xb[k];
+            const float H = voigt_rt((x.x - h) + (x.y - l), tabs, a, H0);
+            if (e0 + lane < values) out[e0 + lane] = ALPHA ? fmaf(ca, H, ct) : H;
+            cell += dcell;
+            k += dk;
+            if (k >= nch) {
+                k -= nch;
+                ++cell;
             }
         }
     }
@@ -254,6 +316,14 @@ __device__ __forceinline__ float2 exp_neg2(float2 x)
 
 // (1 - e^{-d})/d of two values without a branch: from e^{-d} above d = 0.05,
 // else its Taylor series 1 - d/2 + d^2/6 - d^3/24 + d^4/120 (Horner in d)
+__device__ __forceinline__ float2 escape_series2(float2 d)
+{
+    float2 sm = __ffma2_rn(make_float2(1.0f / 120.0f, 1.0f / 120.0f), d, make_float2(-1.0f / 24.0f, -1.0f / 24.0f));
+    sm = __ffma2_rn(sm, d, make_float2(1.0f / 6.0f, 1.0f / 6.0f));
+    sm = __ffma2_rn(sm, d, make_float2(-0.5f, -0.5f));
+    return __ffma2_rn(sm, d, make_float2(1.0f, 1.0f));
+}
+
 __device__ __forceinline__ float2 escape_factor2(float2 d)
 {
     const float2 e = exp_neg2(d);
@@ -261,143 +331,210 @@ __device__ __forceinline__ float2 escape_factor2(float2 d)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd.x) : "f"(d.x));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd.y) : "f"(d.y));
     const float2 lg = __fmul2_rn(sub2(make_float2(1.0f, 1.0f), e), rd);
-    float2 sm = __ffma2_rn(make_float2(1.0f / 120.0f, 1.0f / 120.0f), d, make_float2(-1.0f / 24.0f, -1.0f / 24.0f));
-    sm = __ffma2_rn(sm, d, make_float2(1.0f / 6.0f, 1.0f / 6.0f));
-    sm = __ffma2_rn(sm, d, make_float2(-0.5f, -0.5f));
-    sm = __ffma2_rn(sm, d, make_float2(1.0f, 1.0f));
+    const float2 sm = escape_series2(d);
     return make_float2(d.x > 0.05f ? lg.x : sm.x, d.y > 0.05f ? lg.y : sm.y);
 }
 
-// One cell's extinction and emissivity for a lane's four channels, as two
-// pairs. FULL (n_ch = 4 LPR, rows 16-byte aligned): lane `sub` of a ray holds
-// channels 4 sub .. 4 sub + 3, read as one 16-byte vector per row, so a
-// ray's lanes read each row in one contiguous sweep. Otherwise pair h holds
-// channels sub + LPR (2h) and sub + LPR (2h + 1); channels past n_ch read zeros
-// (dtau = 0 and no intensity).
-template <int LPR, bool FULL>
-__device__ __forceinline__ void cell_rows(const RayArgs& A, int c, int sub, float2 (&v)[2], float2 (&j)[2])
+// CPL (4 or 8) consecutive floats as one read-only vector load.
+template <int CPL>
+__device__ __forceinline__ void read_row(const float* p, float (&r)[CPL])
 {
-    const float* arow = A.hcube + (size_t)c * A.n_ch;
-    const float* jrow = A.emiss + (size_t)c * A.n_ch;
-    if constexpr (FULL) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(arow) + sub);
-        const float4 e = __ldg(reinterpret_cast<const float4*>(jrow) + sub);
-        v[0] = make_float2(a.x, a.y);
-        v[1] = make_float2(a.z, a.w);
-        j[0] = make_float2(e.x, e.y);
-        j[1] = make_float2(e.z, e.w);
+    if constexpr (CPL == 8)
+        asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+            : "l"(p));
+    else
+        asm("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]) : "l"(p));
+}
+
+// One cell's extinction (or profile) and emissivity for CPL channels from k0
+// on, in pairs. VEC (n_ch a multiple of CPL, rows aligned to CPL floats): one
+// 16- or 32-byte vector per row. Otherwise single reads; channels past n_ch read zeros (dtau = 0
+// and no intensity). CPL 1 keeps a zero in its pair's second half.
+template <int CPL, bool VEC>
+__device__ __forceinline__ void cell_rows(const RayArgs& A, int c, int k0, float2 (&v)[(CPL + 1) / 2],
+                                          float2 (&j)[(CPL + 1) / 2])
+{
+    const float* arow = A.hcube + (size_t)c * A.n_ch + k0;
+    const float* jrow = A.emiss + (size_t)c * A.n_ch + k0;
+    if constexpr (VEC) {
+        float a[CPL], e[CPL];
+        read_row<CPL>(arow, a);
+        read_row<CPL>(jrow, e);
+#pragma unroll
+        for (int h = 0; h < CPL / 2; ++h) {
+            v[h] = make_float2(a[2 * h], a[2 * h + 1]);
+            j[h] = make_float2(e[2 * h], e[2 * h + 1]);
+        }
     } else {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int ka = sub + LPR * (2 * h), kb = ka + LPR;
-            v[h] = make_float2(ka < A.n_ch ? __ldg(arow + ka) : 0.0f, kb < A.n_ch ? __ldg(arow + kb) : 0.0f);
-            j[h] = make_float2(ka < A.n_ch ? __ldg(jrow + ka) : 0.0f, kb < A.n_ch ? __ldg(jrow + kb) : 0.0f);
+        for (int h = 0; h < (CPL + 1) / 2; ++h) {
+            const bool a = k0 + 2 * h < A.n_ch, b = CPL > 1 && k0 + 2 * h + 1 < A.n_ch;
+            v[h] = make_float2(a ? __ldg(arow + 2 * h) : 0.0f, b ? __ldg(arow + 2 * h + 1) : 0.0f);
+            j[h] = make_float2(a ? __ldg(jrow + 2 * h) : 0.0f, b ? __ldg(jrow + 2 * h + 1) : 0.0f);
         }
     }
 }
 
-// Channel of element e of pair h of lane `sub` (the layout of cell_rows).
-template <int LPR, bool FULL>
-__device__ __forceinline__ int lane_channel(int sub, int h, int e)
-{
-    return FULL ? 4 * sub + 2 * h + e : sub + LPR * (2 * h + e);
-}
+constexpr int kTileX = 8, kTileY = 4;       // a warp's pixels
+constexpr int kTraceBlock = 128;
 
-// The trace over the per-camera cube (k_rt_profile): LPR lanes per ray, 4
-// channels per lane, so a warp follows 32 / LPR neighbouring rays, whose
-// walks through the grid nearly coincide. The per-segment work (face
-// distances, cell index) is shared by fewer lanes' worth of channels than
-// with one ray per warp. The cube holds the extinction alpha0 H + alpha_abs
-// (JL false) or H (JL true: the line-emission term needs H; alpha is formed
-// here).
-template <int LPR, bool JL, bool FULL>
-__global__ void __launch_bounds__(256, 4) k_trace_cube(const RayArgs A)
+// The trace over the per-camera cube (k_rt_profile). A warp follows the rays
+// of 8 x 4 neighbouring pixels, one per lane, for the same CPL channels; the
+// channel blocks of a tile are neighbouring CTAs. The lanes' cells nearly
+// coincide (pixels oversample the cells), so their reads share sectors and
+// their optical depths are alike: a line a few thermal widths wide touches a
+// block of channels in a small part of the cells, and elsewhere the warp
+// skips, by vote, what does not change the result:
+//   * dtau <= 0.05 in all lanes: (1 - e^{-d})/d is its series, no exponential
+//     or reciprocal; dtau <= 5e-8: the series rounds to 1;
+//   * the optical depths in front did not change: e^{-tau} is the last one's.
+// The values are those of the full formula in every lane. With one ray's 64
+// channels over 16 lanes (every warp has a line-centre lane) the trace of
+// 256^3 cells x 64 channels at 1024^2 pixels took 22.3 ms, bound by issue and
+// special-function slots.
+// The cube holds the extinction alpha0 H + alpha_abs (JL false) or H (JL true:
+// the line-emission term needs H; alpha is formed here).
+template <int CPL, int D, int MINB, bool JL, bool VEC>
+__global__ void __launch_bounds__(kTraceBlock, MINB) k_trace_cube(const RayArgs A, int tiles_x, int blocks_ch)
 {
-    constexpr int CPL = 4;
+    constexpr int HP = (CPL + 1) / 2;
     const int lane = threadIdx.x & 31;
-    const int sub = lane % LPR;
-    const long long ray = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 / LPR) + lane / LPR;
-    const long long npix = (long long)A.npix_x * A.npix_y;
-    if (ray >= npix) return;                 // no warp-wide operations follow
-    const int ix = (int)(ray % A.npix_x);
-    const int iy = (int)(ray / A.npix_x);
+    const int k0 = (int)(blockIdx.x % (unsigned)blocks_ch) * CPL;
+    const long long tile = (long long)(blockIdx.x / (unsigned)blocks_ch) * (kTraceBlock / 32) + (threadIdx.x >> 5);
+    // lanes in Z order: a wide load serves 4 or 8 lanes at a time, which then
+    // are 2 x 2 or 4 x 2 pixels and mostly one cell
+    const int ix = (int)(tile % tiles_x) * kTileX + ((lane & 1) | (lane >> 1 & 2) | (lane >> 2 & 4));
+    const long long iyl = tile / tiles_x * kTileY + ((lane >> 1 & 1) | (lane >> 2 & 2));
+    const bool pixel = ix < A.npix_x && iyl < A.npix_y;
+    const int iy = (int)iyl;
 
-    // the ray's start (k_ray_setup): first cell, position in it, hit
-    const float4 r0 = __ldg(A.rayinit + 2 * ray), r1 = __ldg(A.rayinit + 2 * ray + 1);
     // the lane's channel pairs: intensity, optical depth in front of the
-    // segment, and their compensation terms
-    float2 I[CPL / 2], Ic[CPL / 2], tau[CPL / 2], tc[CPL / 2];
+    // segment, their compensation terms, and e^{-tau}
+    float2 I[HP], Ic[HP], tau[HP], tc[HP], T[HP];
 #pragma unroll
-    for (int h = 0; h < CPL / 2; ++h) I[h] = Ic[h] = tau[h] = tc[h] = make_float2(0.0f, 0.0f);
-
-    if (__float_as_int(r0.w)) {
-        // cell and in-cell position as scalars (an array indexed by the
-        // crossing axis would live in local memory); the crossing axis is
-        // applied by selects
-        int ci0 = __float_as_int(r0.x), ci1 = __float_as_int(r0.y), ci2 = __float_as_int(r0.z);
-        float p0 = r1.x, p1 = r1.y, p2 = r1.z;
-        const float d0 = A.dirf[0], d1 = A.dirf[1], d2 = A.dirf[2];
-        const int nx = A.nx, ny = A.ny, nz = A.nz, nxy = A.nx * A.ny;
+    for (int h = 0; h < HP; ++h) {
+        I[h] = Ic[h] = tau[h] = tc[h] = make_float2(0.0f, 0.0f);
+        T[h] = make_float2(1.0f, 1.0f);
+    }
+    // the ray's start (k_ray_setup): first cell, position in it, hit. What
+    // depends on the axis of a crossing is applied by selects (an array
+    // indexed by it would live in local memory): the signed cell stride, the
+    // side a cell is entered on, and the cells left before the box's face.
+    int r0 = 0, r1 = 0, r2 = 0, c = 0;
+    bool on = false;
+    float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f;
+    const float d0 = A.dirf[0], d1 = A.dirf[1], d2 = A.dirf[2];
+    const bool f0 = d0 > 0.0f, f1 = d1 > 0.0f, f2 = d2 > 0.0f;
+    const int st0 = f0 ? 1 : -1, st1 = f1 ? A.nx : -A.nx, st2 = f2 ? A.nx * A.ny : -A.nx * A.ny;
+    const float e0 = f0 ? 0.0f : 1.0f, e1 = f1 ? 0.0f : 1.0f, e2 = f2 ? 0.0f : 1.0f;
+    if (pixel) {
+        const long long ray = (long long)iy * A.npix_x + ix;
+        const float4 q0 = __ldg(A.rayinit + 2 * ray), q1 = __ldg(A.rayinit + 2 * ray + 1);
+        const int c0 = __float_as_int(q0.x), c1 = __float_as_int(q0.y), c2 = __float_as_int(q0.z);
+        p0 = q1.x;
+        p1 = q1.y;
+        p2 = q1.z;
         // the ray's start can lie outside (a ray along the box's face); after
         // that only the axis just stepped on can leave the box
-        const bool inside = ci0 >= 0 && ci0 < nx && ci1 >= 0 && ci1 < ny && ci2 >= 0 && ci2 < nz;
-        const unsigned fwd = (d0 > 0.0f ? 1u : 0u) | (d1 > 0.0f ? 2u : 0u) | (d2 > 0.0f ? 4u : 0u);
-        const int max_seg = inside ? nx + ny + nz + 3 : 0;
-        int c = (ci2 * ny + ci1) * nx + ci0;
-        for (int seg = 0; seg < max_seg; ++seg) {
-            // distance to the face ahead on each axis, one FMA each
-            float s = fmaf(p0, A.face_neg[0], A.face_c[0]);
-            int axis = 0;
-            const float t1 = fmaf(p1, A.face_neg[1], A.face_c[1]);
-            if (t1 < s) { s = t1; axis = 1; }
-            const float t2 = fmaf(p2, A.face_neg[2], A.face_c[2]);
-            if (t2 < s) { s = t2; axis = 2; }
-            float2 v[2], j[2];
-            cell_rows<LPR, FULL>(A, c, sub, v, j);
-            float a0 = 0.0f, ta = 0.0f, jl = 0.0f;
-            if (JL) {
-                a0 = __ldg(A.cells + c).x;
-                ta = A.tau_abs ? __ldg(A.tau_abs + c) : 0.0f;
-                jl = __ldg(A.jline + c) * 0.56418958354775628f;
-            }
-            const float2 s2 = make_float2(s, s);
-#pragma unroll
-            for (int h = 0; h < CPL / 2; ++h) {
-                float2 vv = v[h], jj = j[h];
-                if (JL) {
-                    jj = __ffma2_rn(make_float2(jl, jl), vv, jj);
-                    vv = __ffma2_rn(make_float2(a0, a0), vv, make_float2(ta, ta));
-                }
-                const float2 dtau = __fmul2_rn(vv, s2);
-                const float2 T = exp_neg2(tau[h]);
-                kahan_add2(I[h], Ic[h], __fmul2_rn(__fmul2_rn(__fmul2_rn(T, jj), s2), escape_factor2(dtau)));
-                kahan_add2(tau[h], tc[h], dtau);
-            }
-            // move to the face, then step across it (the crossing axis is set exactly)
-            p0 = __saturatef(fmaf(s, d0, p0));
-            p1 = __saturatef(fmaf(s, d1, p1));
-            p2 = __saturatef(fmaf(s, d2, p2));
-            const bool x0 = axis == 0, x1 = axis == 1;
-            const bool up = (fwd >> axis) & 1u;
-            const int nc = (x0 ? ci0 : (x1 ? ci1 : ci2)) + (up ? 1 : -1);
-            const int dim = x0 ? nx : (x1 ? ny : nz);
-            if ((unsigned)nc >= (unsigned)dim) break;
-            const float pn = up ? 0.0f : 1.0f;
-            ci0 = x0 ? nc : ci0;
-            ci1 = x1 ? nc : ci1;
-            ci2 = (x0 || x1) ? ci2 : nc;
-            p0 = x0 ? pn : p0;
-            p1 = x1 ? pn : p1;
-            p2 = (x0 || x1) ? p2 : pn;
-            const int stride = x0 ? 1 : (x1 ? nx : nxy);
-            c += up ? stride : -stride;
+        on = __float_as_int(q0.w) && c0 >= 0 && c0 < A.nx && c1 >= 0 && c1 < A.ny && c2 >= 0 && c2 < A.nz;
+        if (on) {
+            c = (c2 * A.ny + c1) * A.nx + c0;
+            r0 = f0 ? A.nx - 1 - c0 : c0;
+            r1 = f1 ? A.ny - 1 - c1 : c1;
+            r2 = f2 ? A.nz - 1 - c2 : c2;
         }
     }
+    // The geometry does not depend on what is read: a ray marches D segments
+    // ahead and requests their rows together.
+    while (__any_sync(0xffffffffu, on)) {
+        float2 vq[D][HP], jq[D][HP];
+        float sq[D], tq[D];
+        float2 lq[D];           // JL: {alpha0, jline / sqrt(pi)}, tq the continuum
+        bool oq[D];
 #pragma unroll
-    for (int h = 0; h < CPL / 2; ++h) {
-        const int ka = lane_channel<LPR, FULL>(sub, h, 0), kb = lane_channel<LPR, FULL>(sub, h, 1);
-        if (ka < A.n_ch) A.maps[((size_t)ka * A.npix_y + iy) * A.npix_x + ix] = I[h].x;
-        if (kb < A.n_ch) A.maps[((size_t)kb * A.npix_y + iy) * A.npix_x + ix] = I[h].y;
+        for (int q = 0; q < D; ++q) {
+            oq[q] = on;
+            if (on) {
+                cell_rows<CPL, VEC>(A, c, k0, vq[q], jq[q]);
+                if (JL) {
+                    lq[q] = make_float2(__ldg(A.cells + c).x, __ldg(A.jline + c) * 0.56418958354775628f);
+                    tq[q] = A.tau_abs ? __ldg(A.tau_abs + c) : 0.0f;
+                }
+            }
+            // distance to the face ahead on each axis, one FMA each
+            float s = fmaf(p0, A.face_neg[0], A.face_c[0]);
+            const float t1 = fmaf(p1, A.face_neg[1], A.face_c[1]);
+            const float t2 = fmaf(p2, A.face_neg[2], A.face_c[2]);
+            bool x0 = true, x1 = false, x2 = false;
+            if (t1 < s) { s = t1; x0 = false; x1 = true; }
+            if (t2 < s) { s = t2; x0 = false; x1 = false; x2 = true; }
+            sq[q] = s;
+            // move to the face, then step across it (the crossing axis is set exactly)
+            p0 = x0 ? e0 : __saturatef(fmaf(s, d0, p0));
+            p1 = x1 ? e1 : __saturatef(fmaf(s, d1, p1));
+            p2 = x2 ? e2 : __saturatef(fmaf(s, d2, p2));
+            c += x0 ? st0 : (x1 ? st1 : st2);
+            r0 -= x0 ? 1 : 0;
+            r1 -= x1 ? 1 : 0;
+            r2 -= x2 ? 1 : 0;
+            on = on && (r0 | r1 | r2) >= 0;
+        }
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+        if (D > 1 && q > 0 && !__any_sync(0xffffffffu, oq[q])) break;
+        const bool now = oq[q];
+        float2 v[HP], j[HP];
+#pragma unroll
+        for (int h = 0; h < HP; ++h) {
+            v[h] = now ? vq[q][h] : make_float2(0.0f, 0.0f);
+            j[h] = now ? jq[q][h] : make_float2(0.0f, 0.0f);
+            if (JL && now) {
+                j[h] = __ffma2_rn(make_float2(lq[q].y, lq[q].y), v[h], j[h]);
+                v[h] = __ffma2_rn(make_float2(lq[q].x, lq[q].x), v[h], make_float2(tq[q], tq[q]));
+            }
+        }
+        const float2 s2 = make_float2(sq[q], sq[q]);
+        float2 dt[HP];
+        float dmax = 0.0f;
+#pragma unroll
+        for (int h = 0; h < HP; ++h) {
+            dt[h] = __fmul2_rn(v[h], s2);
+            dmax = fmaxf(dmax, fmaxf(dt[h].x, dt[h].y));
+        }
+        float2 tj[HP];          // T j s
+#pragma unroll
+        for (int h = 0; h < HP; ++h) tj[h] = __fmul2_rn(__fmul2_rn(T[h], j[h]), s2);
+        if (__any_sync(0xffffffffu, dmax > 5e-8f)) {            // warp-uniform
+            if (__any_sync(0xffffffffu, dmax > 0.05f)) {
+#pragma unroll
+                for (int h = 0; h < HP; ++h) tj[h] = __fmul2_rn(tj[h], escape_factor2(dt[h]));
+            } else {
+#pragma unroll
+                for (int h = 0; h < HP; ++h) tj[h] = __fmul2_rn(tj[h], escape_series2(dt[h]));
+            }
+        }
+        bool moved = false;
+        if (now) {
+#pragma unroll
+            for (int h = 0; h < HP; ++h) {
+                kahan_add2(I[h], Ic[h], tj[h]);
+                const float2 before = tau[h];
+                kahan_add2(tau[h], tc[h], dt[h]);
+                moved = moved || tau[h].x != before.x || tau[h].y != before.y;
+            }
+        }
+        if (__any_sync(0xffffffffu, moved)) {
+#pragma unroll
+            for (int h = 0; h < HP; ++h) T[h] = exp_neg2(tau[h]);
+        }
+        }
+    }
+    if (pixel) {
+#pragma unroll
+        for (int e = 0; e < CPL; ++e)
+            if (k0 + e < A.n_ch)
+                A.maps[((size_t)(k0 + e) * A.npix_y + iy) * A.npix_x + ix] = e & 1 ? I[e / 2].y : I[e / 2].x;
     }
 }
 
@@ -406,17 +543,8 @@ __global__ void __launch_bounds__(256, 4) k_trace_cube(const RayArgs A)
 template <int CPL>
 __global__ void __launch_bounds__(256) k_raytrace(const RayArgs A)
 {
-    __shared__ float sv[kVoigtN];
-    __shared__ int eI[kRtEn];
-    __shared__ float eF[kRtEn];
-    for (int i = threadIdx.x; i < kVoigtN; i += blockDim.x) sv[i] = A.voigt_lnH[i];
-    if (threadIdx.x < kRtEn) {
-        const double t = (double)((kVoigtN - 1) / (kVoigtL1 - kVoigtL0)) *
-                         (((int)threadIdx.x + kRtEmin) * 0.30102999566398119521 - kVoigtL0);
-        const double it = floor(t);
-        eI[threadIdx.x] = (int)it;
-        eF[threadIdx.x] = (float)(t - it);
-    }
+    __shared__ ProfileTables tabs;
+    load_tables(tabs, A.voigt_lnH);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -473,11 +601,7 @@ __global__ void __launch_bounds__(256) k_raytrace(const RayArgs A)
             p[d] = (float)r;
             inv[d] = 1.0f / dir[d];
         }
-        float nh[3], nl[3];
-        for (int d = 0; d < 3; ++d) {
-            nh[d] = (float)n[d];
-            nl[d] = (float)(n[d] - (double)nh[d]);
-        }
+        const float nh[3] = {A.nh[0], A.nh[1], A.nh[2]}, nl[3] = {A.nl[0], A.nl[1], A.nl[2]};
         const int max_seg = A.nx + A.ny + A.nz + 3;
         for (int seg = 0; seg < max_seg; ++seg) {
             if (ci[0] < 0 || ci[0] >= A.nx || ci[1] < 0 || ci[1] >= A.ny || ci[2] < 0 || ci[2] >= A.nz) break;
@@ -500,7 +624,7 @@ __global__ void __launch_bounds__(256) k_raytrace(const RayArgs A)
                 const int k = lane + 32 * q;
                 if (k < A.n_ch) {
                     const float xk = (xbh[q] - vnh) + (xbl[q] - vnl);
-                    const float H = voigt_rt(xk, sv, eI, eF, a, H0);
+                    const float H = voigt_rt(xk, tabs, a, H0);
                     const float dtau = fmaf(rec.x, H, ta) * s;
                     float j = __ldg(jrow + k);
                     if (A.jline) j = fmaf(jl * 0.56418958354775628f, H, j);
@@ -525,45 +649,74 @@ __global__ void __launch_bounds__(256) k_raytrace(const RayArgs A)
 
 }  // namespace
 
-// The profile cube (when A.hcube), then the trace over it with LPR lanes
-// per ray; without the cube, the one-ray-per-warp trace that evaluates the
-// profile per segment.
-template <int CPL, int LPR>
+template <int CPL, int D, int MINB, bool VEC>
+cudaError_t launch_trace(const RayArgs& A, cudaStream_t s)
+{
+    const int tiles_x = (A.npix_x + kTileX - 1) / kTileX;
+    const long long tiles = (long long)tiles_x * ((A.npix_y + kTileY - 1) / kTileY);
+    const int blocks_ch = (A.n_ch + CPL - 1) / CPL;
+    const long long blocks = (tiles + kTraceBlock / 32 - 1) / (kTraceBlock / 32) * blocks_ch;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    if (A.jline) k_trace_cube<CPL, D, MINB - (CPL == 8 && VEC ? 1 : 0), true, VEC><<<(unsigned)blocks, kTraceBlock, 0, s>>>(A, tiles_x, blocks_ch);
+    else k_trace_cube<CPL, D, MINB, false, VEC><<<(unsigned)blocks, kTraceBlock, 0, s>>>(A, tiles_x, blocks_ch);
+    return cudaGetLastError();
+}
+
+// Channels per lane: the most of 8, 4, 2, 1 that pad the channels by at most
+// a quarter and leave enough lanes to hide the latency of the reads, about 50
+// warps per SM (fewer channels per lane repeat the geometry's work for more
+// lanes). Measured, us per call with profile cube: 1024^2 pixels x 64
+// channels x 256^3 cells 19.5 with 8 (22.2 with 4, in ms); 400^2 x 16 x 128^3
+// 633 / 655 / 1040 with 8 / 4 / 2; 256^2 x 10 x 64^3 228 / 174 / 166 / 226
+// with 8 / 4 / 2 / 1; 128^2 x 5 x 128^3 264 / 252 / 203 / 179.
+cudaError_t launch_trace_any(const RayArgs& A, int sm_count, cudaStream_t s)
+{
+    const long long npix = (long long)A.npix_x * A.npix_y, enough = (long long)sm_count * 1640;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(A.emiss) | reinterpret_cast<uintptr_t>(A.hcube);
+    auto fits = [&](int cpl) {
+        const int nb = (A.n_ch + cpl - 1) / cpl;
+        return 4 * nb * cpl <= 5 * A.n_ch && npix * nb >= enough;
+    };
+    if (fits(8)) {
+        if (A.n_ch % 8 == 0 && (at & 31u) == 0) return launch_trace<8, 2, 5, true>(A, s);
+        if (A.n_ch % 4 || (at & 15u)) return launch_trace<8, 2, 4, false>(A, s);
+    }
+    if (fits(4)) {
+        if (A.n_ch % 4 == 0 && (at & 15u) == 0) return launch_trace<4, 2, 6, true>(A, s);
+        return launch_trace<4, 2, 6, false>(A, s);
+    }
+    if (fits(2)) return launch_trace<2, 4, 8, false>(A, s);
+    return launch_trace<1, 4, 8, false>(A, s);
+}
+
+// The profile cube (when A.hcube), then the trace over it; without the cube,
+// the one-ray-per-warp trace that evaluates the profile per segment.
+template <int CPL>
 cudaError_t launch_cpl(const RayArgs& A, int sm_count, cudaStream_t s)
 {
     const long long npix = (long long)A.npix_x * A.npix_y;
     if (A.hcube) {
-        const long long blocks = (npix * LPR + 255) / 256;
-        if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
         k_ray_setup<<<(unsigned)((npix + 255) / 256), 256, 0, s>>>(A);
-        // the vector reads need each lane's four channels 16-byte aligned
-        const bool full = A.n_ch == 4 * LPR && (reinterpret_cast<uintptr_t>(A.emiss) & 15u) == 0 &&
-                          (reinterpret_cast<uintptr_t>(A.hcube) & 15u) == 0;
-        if (A.jline) {
-            k_rt_profile<CPL, false><<<sm_count * 8, 256, 0, s>>>(A, A.hcube);
-            if (full) k_trace_cube<LPR, true, true><<<(unsigned)blocks, 256, 0, s>>>(A);
-            else k_trace_cube<LPR, true, false><<<(unsigned)blocks, 256, 0, s>>>(A);
+        if (A.n_ch % 32) {
+            if (A.jline) k_rt_profile_flat<false><<<sm_count * 8, 256, 0, s>>>(A, A.hcube);
+            else k_rt_profile_flat<true><<<sm_count * 8, 256, 0, s>>>(A, A.hcube);
         } else {
-            k_rt_profile<CPL, true><<<sm_count * 8, 256, 0, s>>>(A, A.hcube);
-            if (full) k_trace_cube<LPR, false, true><<<(unsigned)blocks, 256, 0, s>>>(A);
-            else k_trace_cube<LPR, false, false><<<(unsigned)blocks, 256, 0, s>>>(A);
+            if (A.jline) k_rt_profile<CPL, false><<<sm_count * 8, 256, 0, s>>>(A, A.hcube);
+            else k_rt_profile<CPL, true><<<sm_count * 8, 256, 0, s>>>(A, A.hcube);
         }
-    } else {
-        const long long blocks = (npix * 32 + 255) / 256;
-        if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-        k_raytrace<CPL><<<(unsigned)blocks, 256, 0, s>>>(A);
+        return launch_trace_any(A, sm_count, s);
     }
+    const long long blocks = (npix * 32 + 255) / 256;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    k_raytrace<CPL><<<(unsigned)blocks, 256, 0, s>>>(A);
     return cudaGetLastError();
 }
 
 cudaError_t launch_raytrace(const RayArgs& A, int sm_count, cudaStream_t s)
 {
-    if (A.n_ch <= 4) return launch_cpl<1, 1>(A, sm_count, s);
-    if (A.n_ch <= 8) return launch_cpl<1, 2>(A, sm_count, s);
-    if (A.n_ch <= 16) return launch_cpl<1, 4>(A, sm_count, s);
-    if (A.n_ch <= 32) return launch_cpl<1, 8>(A, sm_count, s);
-    if (A.n_ch <= 64) return launch_cpl<2, 16>(A, sm_count, s);
-    if (A.n_ch <= 128) return launch_cpl<4, 32>(A, sm_count, s);
+    if (A.n_ch <= 32) return launch_cpl<1>(A, sm_count, s);
+    if (A.n_ch <= 64) return launch_cpl<2>(A, sm_count, s);
+    if (A.n_ch <= 128) return launch_cpl<4>(A, sm_count, s);
     return cudaErrorInvalidValue;
 }
 
