@@ -63,7 +63,9 @@ constexpr size_t kSmemBytes = (size_t)kSmemRowBins + 2 * kRowGuideN * 16 + kUsNx
 enum : unsigned {
     F_VEL = 1u,       // cells carry a bulk velocity
     F_SCAT = 2u,      // per-cell scattering counts
-    F_RICH = 4u,      // excitation / mean intensity / emissivity / destruction
+    F_RICH = 4u,      // any of excitation, mean intensity, emissivity, destruction, continuum
+    F_SEG = 8u,       // (with F_RICH) mean intensity or emissivity: tallies of every segment
+    F_WIDE = 16u,     // (with F_RICH, without F_SEG) in the larger CTA, transport_light_block()
 };
 
 enum { ST_EMITTED = 0, ST_ESCAPED, ST_DESTROYED, ST_STUCK, ST_SCAT, ST_CROSS, ST_ABSORBED, ST_N = 8 };
@@ -198,6 +200,8 @@ cudaError_t launch_transport_ph(const TransportArgs& A, int ph_mode, int precisi
 int transport_occupancy_ph(int ph_mode, int precision, unsigned features, int block);
 // Largest CTA the instantiation is compiled for (512 lean FP32, else 256).
 int transport_max_block(int precision, unsigned features);
+// CTA of the F_WIDE walk (FP32, profile mode 2).
+int transport_light_block();
 // The batched launch: its CTA size limit and occupancy.
 int transport_batch_max_block();
 int transport_batch_occupancy(int precision, unsigned features, int block);

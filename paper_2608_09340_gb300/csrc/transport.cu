@@ -45,6 +45,8 @@ int transport_max_block(int precision, unsigned features)
     return (precision == KRL_PREC_FP32 && !(features & F_RICH)) ? 512 : 256;
 }
 
+int transport_light_block() { return kLightBlock; }
+
 int transport_occupancy(int precision, unsigned features, int block, int ph_mode)
 {
     if (ph_mode == 1 || ph_mode == 3 || ph_mode == 4) return transport_occupancy_ph(ph_mode, precision, features, block);

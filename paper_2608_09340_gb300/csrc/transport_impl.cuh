@@ -37,6 +37,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "krl_internal.cuh"
 
 namespace krl {
@@ -456,7 +458,8 @@ __device__ __forceinline__ int us_bin(R xi, R& L)
 
 // Per-lane event counters (summed over the CTA at the end of a model).
 struct LaneStats {
-    unsigned long long emit, esc, des, stuck, scat, cross, absorbed;
+    unsigned esc, des, stuck, absorbed;     // packets of one lane (every emitted one ends in one of these)
+    unsigned scat, cross;                   // kept below 2^31 (end_packet)
 };
 
 template <typename R>
@@ -467,7 +470,7 @@ struct Pkt {
     R ix, iy, iz;          // 1 / n
     R x, tau;
     float4 rec;            // current cell record
-    uint32_t nscat, ncross, cell0;
+    uint32_t nscat, ncross;
     unsigned long long id;
     uint32_t vis_scat;     // scatterings in this cell visit
     R vis_exc;             // sum w ds H over this cell visit
@@ -560,15 +563,13 @@ template <typename R>
 __device__ __forceinline__ void write_record(const TransportArgs& A, const Pkt<R>& p, uint16_t status)
 {
     if (!A.rec) return;
-    krl_packet_record r;
+    krl_packet_record& r = A.rec[p.id - A.first];       // (cell0 is written at emission)
     r.x = (float)p.x;
     r.nscat = p.nscat;
     r.ncross = p.ncross;
     r.status = status;
     r.pad = 0;
-    r.cell0 = p.cell0;
     r.scat_cells = sizeof(R) == 8 ? p.cellsum : 0u;
-    A.rec[p.id - A.first] = r;
 }
 
 // X = dim u, u = (2 (r >> 9) + 1) 2^-24 the uniform of word r: the product is
@@ -707,7 +708,7 @@ __device__ __forceinline__ bool emit(const TransportArgs& A, const RoundKeys& K,
     p.prev_scat = true;
     if (!inside) {
         p.x = xcom;
-        p.cell0 = 0xFFFFFFFFu;
+        if (A.rec) A.rec[p.id - A.first].cell0 = 0xFFFFFFFFu;
         return false;
     }
     p.cx = ci[0];
@@ -717,7 +718,7 @@ __device__ __forceinline__ bool emit(const TransportArgs& A, const RoundKeys& K,
     p.py = pp[1];
     p.pz = pp[2];
     p.c = (ci[2] * A.ny + ci[1]) * A.nx + ci[0];
-    p.cell0 = (uint32_t)p.c;
+    if (A.rec) A.rec[p.id - A.first].cell0 = (uint32_t)p.c;
     p.rec = __ldg(A.cells + p.c);
     R vdn = (F & F_VEL) ? vdot<R>(p.nx, p.ny, p.nz, p.rec) : (R)0;
     p.x = xcom + vdn;
@@ -1004,11 +1005,19 @@ __device__ __forceinline__ T warp_sum(T v)
     return v;
 }
 
-// Launch shape per instantiation: the lean FP32 walk runs 512-thread CTAs,
-// two per SM (64 registers each); the FP64 and rich-tally walks need more
-// registers and run 256-thread CTAs.
+// Launch shape per instantiation, two CTAs per SM each: the lean FP32 walk
+// runs 512-thread CTAs (64 registers each), the FP32 walk with weights,
+// destruction or excitation but no per-segment tallies 384 (F_WIDE, 80
+// registers) or 256, the others, which need more registers, 256. Shared memory holds two CTAs'
+// tables, so more warps per SM mean larger CTAs. On the 128^3 cloud (86 events
+// per packet, 16 warps per SM issued in half the cycles) 384 threads took the
+// Lambda cycle from 79 to 66 ms, 512 (with spills) 75.
+constexpr int kLightBlock = 384;
 template <typename R, unsigned F>
-constexpr int max_block() { return (sizeof(R) == 4 && !(F & F_RICH)) ? 512 : 256; }
+constexpr int max_block()
+{
+    return sizeof(R) == 8 || (F & F_RICH) ? ((F & F_WIDE) ? kLightBlock : 256) : 512;
+}
 
 // ---------------------------------------------------------------- tail compaction
 //
@@ -1025,11 +1034,11 @@ constexpr int kTailRound = 32;
 // with no idle lane.
 constexpr int kBulkCheck = 16;
 
-// Words per stashed packet: cell (c, cx, cy, cz), nscat, ncross, cell0, id
+// Words per stashed packet: cell (c, cx, cy, cz), nscat, ncross, id
 // (2 words), the scattering-cell sum (FP64 walk), and px, py, pz, nx, ny, nz,
 // x, tau (and the weight in the rich walk) in R.
 template <typename R, unsigned F>
-constexpr int stash_words() { return 9 + (sizeof(R) == 8 ? 1 : 0) + ((F & F_RICH) ? 9 : 8) * (int)(sizeof(R) / 4); }
+constexpr int stash_words() { return 8 + (sizeof(R) == 8 ? 1 : 0) + ((F & F_RICH) ? 9 : 8) * (int)(sizeof(R) / 4); }
 
 // (the stash, or the buffers of the last packets' walk in its place)
 template <typename R, unsigned F>
@@ -1073,7 +1082,6 @@ __device__ __forceinline__ void stash_put(uint32_t* w, int n, int slot, const Pk
     w[(f++) * n + slot] = (uint32_t)p.cz;
     w[(f++) * n + slot] = p.nscat;
     w[(f++) * n + slot] = p.ncross;
-    w[(f++) * n + slot] = p.cell0;
     w[(f++) * n + slot] = (uint32_t)p.id;
     w[(f++) * n + slot] = (uint32_t)(p.id >> 32);
     if constexpr (sizeof(R) == 8) w[(f++) * n + slot] = p.cellsum;
@@ -1098,7 +1106,6 @@ __device__ __forceinline__ void stash_get(const TransportArgs& A, const uint32_t
     p.cz = (int)w[(f++) * n + slot];
     p.nscat = w[(f++) * n + slot];
     p.ncross = w[(f++) * n + slot];
-    p.cell0 = w[(f++) * n + slot];
     const uint32_t lo = w[(f++) * n + slot];
     const uint32_t hi = w[(f++) * n + slot];
     p.id = ((unsigned long long)hi << 32) | lo;
@@ -1169,11 +1176,17 @@ __device__ __forceinline__ float to_face(Pkt<float>& p, int& axis, float& nd)
 // A packet's end: status 1 escaped, 2 destroyed, 3 budget, 4 absorbed.
 template <typename R>
 __device__ __forceinline__ void end_packet(const TransportArgs& A, const Pkt<R>& p, uint16_t status,
-                                           unsigned long long& counter, LaneStats& st)
+                                           unsigned& counter, LaneStats& st)
 {
     ++counter;
-    st.scat += p.nscat;
-    st.cross += p.ncross;
+    if ((p.nscat | p.ncross | st.scat | st.cross) >> 30) {      // counts in 32 bits only while the sums fit
+        atomicAdd(A.stats + ST_SCAT, (unsigned long long)st.scat + p.nscat);
+        atomicAdd(A.stats + ST_CROSS, (unsigned long long)st.cross + p.ncross);
+        st.scat = st.cross = 0u;
+    } else {
+        st.scat += p.nscat;
+        st.cross += p.ncross;
+    }
     write_record(A, p, status);
 }
 
@@ -1314,7 +1327,7 @@ __device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys&
         R wseg = p.wgt, ab = (R)0;
         if (A.tau_abs) wseg = p.wgt * seg_factor<R>((R)__ldg(A.tau_abs + p.c) * ds, ab);
         if (A.rich & KRL_TALLY_EXC) p.vis_exc = fma(wseg * ds, H, p.vis_exc);
-        if (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)) rich_segment<R, F>(A, T, p.c, p.rec, p.nx, p.ny, p.nz, ds, xcom, H, wseg);
+        if ((F & F_SEG) && (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS))) rich_segment<R, F>(A, T, p.c, p.rec, p.nx, p.ny, p.nz, ds, xcom, H, wseg);
         if (A.tau_abs) {
             p.vis_abs = fma(p.wgt, ab, p.vis_abs);
             p.wgt = p.wgt * ((R)1 - ab);
@@ -1476,7 +1489,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
     const int nwarps = (int)(blockDim.x >> 5);
     Pkt<R> p;
     bool active = false;
-    LaneStats st = {0, 0, 0, 0, 0, 0, 0};
+    LaneStats st = {0u, 0u, 0u, 0u, 0u, 0u};
 
     // Both phases run in one loop so that the event code is inlined once.
     const int n = (int)blockDim.x;
@@ -1530,7 +1543,6 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
                     const unsigned long long k = base + __popc(idle & ((1u << lane) - 1u));
                     if (k < top) {
                         p.id = A.first + k;
-                        ++st.emit;
                         if (emit<R, F>(A, K, p)) {
                             active = true;
                         } else {
@@ -1563,7 +1575,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
             if (total == 0) break;            // CTA-uniform
             if constexpr (sizeof(R) == 4 && (PH == 2 || PH == 4)) {
                 const int tw = nwarps < kTailWarps ? nwarps : kTailWarps;
-                if (total <= tw * kTailPerWarp && 2 * scatters > total) {     // CTA-uniform
+                if (tail_starts(total, tw) && 2 * scatters > total) {     // CTA-uniform
                     // the last packets, dealt over tw warps: group g of warp
                     // w walks packet g tw + w
                     if (active) {
@@ -1571,7 +1583,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
                         stash_put<R, F>(stash, n, before + __popc(m & ((1u << lane) - 1u)), p);
                     }
                     __syncthreads();
-                    constexpr int G = 32 / kTailPerWarp;
+                    const int G = total <= tw * kTailWide ? 32 / kTailWide : 16 / kTailWide;
                     const int q = (int)lane / G * tw + warp;
                     active = warp < tw && q < total;
                     if (active) stash_get<R, F>(A, stash, n, q, p);
@@ -1601,7 +1613,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
         if (active) active = advance<R, F, PH>(A, K, p, T, a, H0, st);
     }
 
-    if constexpr (sizeof(R) == 4 && (F & F_RICH) != 0) {
+    if constexpr (sizeof(R) == 4 && (F & F_SEG) != 0) {
         // the rest of the warp's last chunk of segment records
         if (A.seg && A.seg_chunk) {
             __syncwarp();
@@ -1610,9 +1622,10 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
             for (unsigned k = lane; k < left; k += 32u) clear_segments(A, i + k, 1u);
         }
     }
-    const unsigned long long tot[7] = {warp_sum(st.emit),  warp_sum(st.esc),  warp_sum(st.des),
-                                       warp_sum(st.stuck), warp_sum(st.scat), warp_sum(st.cross),
-                                       warp_sum(st.absorbed)};
+    using u64 = unsigned long long;
+    const u64 ended = (u64)st.esc + st.des + st.stuck + st.absorbed;
+    const u64 tot[7] = {warp_sum(ended),        warp_sum((u64)st.esc),   warp_sum((u64)st.des),     warp_sum((u64)st.stuck),
+                        warp_sum((u64)st.scat), warp_sum((u64)st.cross), warp_sum((u64)st.absorbed)};
     if (lane == 0) {
 #pragma unroll
         for (int k = 0; k < 7; ++k)
@@ -1712,21 +1725,6 @@ int occupancy_one(int block)
     return n;
 }
 
-template <typename R, int PH>
-cudaError_t dispatch(const TransportArgs& A, unsigned f, int grid, int block, cudaStream_t s)
-{
-    switch (f & 7u) {
-    case 0: return launch_one<R, 0, PH>(A, grid, block, s);
-    case 1: return launch_one<R, 1, PH>(A, grid, block, s);
-    case 2: return launch_one<R, 2, PH>(A, grid, block, s);
-    case 3: return launch_one<R, 3, PH>(A, grid, block, s);
-    case 4: return launch_one<R, 4, PH>(A, grid, block, s);
-    case 5: return launch_one<R, 5, PH>(A, grid, block, s);
-    case 6: return launch_one<R, 6, PH>(A, grid, block, s);
-    default: return launch_one<R, 7, PH>(A, grid, block, s);
-    }
-}
-
 template <typename R, unsigned F>
 int batch_occupancy_one(int block)
 {
@@ -1738,49 +1736,64 @@ int batch_occupancy_one(int block)
     return n;
 }
 
-template <typename R>
-int batch_occ_dispatch(unsigned f, int block)
+// Calls fn with the instantiation of the features f. The walk without
+// per-segment tallies has instantiations of its own in the FP32 production
+// walk only (SPLIT); elsewhere the rich walk handles all of them.
+template <bool SPLIT, typename Fn>
+auto with_features(unsigned f, Fn fn)
 {
+    using std::integral_constant;
+    if constexpr (SPLIT) {
+        constexpr unsigned W = F_RICH | F_WIDE;
+        switch (f & (F_RICH | F_SEG | F_WIDE | 3u)) {
+        case F_RICH: return fn(integral_constant<unsigned, F_RICH>());
+        case F_RICH | 1u: return fn(integral_constant<unsigned, F_RICH | 1u>());
+        case F_RICH | 2u: return fn(integral_constant<unsigned, F_RICH | 2u>());
+        case F_RICH | 3u: return fn(integral_constant<unsigned, F_RICH | 3u>());
+        case W: return fn(integral_constant<unsigned, W>());
+        case W | 1u: return fn(integral_constant<unsigned, W | 1u>());
+        case W | 2u: return fn(integral_constant<unsigned, W | 2u>());
+        case W | 3u: return fn(integral_constant<unsigned, W | 3u>());
+        default: break;
+        }
+    }
     switch (f & 7u) {
-    case 0: return batch_occupancy_one<R, 0>(block);
-    case 1: return batch_occupancy_one<R, 1>(block);
-    case 2: return batch_occupancy_one<R, 2>(block);
-    case 3: return batch_occupancy_one<R, 3>(block);
-    case 4: return batch_occupancy_one<R, 4>(block);
-    case 5: return batch_occupancy_one<R, 5>(block);
-    case 6: return batch_occupancy_one<R, 6>(block);
-    default: return batch_occupancy_one<R, 7>(block);
+    case 0: return fn(integral_constant<unsigned, 0u>());
+    case 1: return fn(integral_constant<unsigned, 1u>());
+    case 2: return fn(integral_constant<unsigned, 2u>());
+    case 3: return fn(integral_constant<unsigned, 3u>());
+    case 4: return fn(integral_constant<unsigned, F_RICH | F_SEG>());
+    case 5: return fn(integral_constant<unsigned, F_RICH | F_SEG | 1u>());
+    case 6: return fn(integral_constant<unsigned, F_RICH | F_SEG | 2u>());
+    default: return fn(integral_constant<unsigned, F_RICH | F_SEG | 3u>());
     }
 }
 
-template <typename R>
-cudaError_t dispatch_batch(const BatchArgs& B, unsigned f, int grid, int block, cudaStream_t s)
+template <typename R, int PH>
+constexpr bool split_rich() { return sizeof(R) == 4 && PH == 2; }
+
+template <typename R, int PH>
+cudaError_t dispatch(const TransportArgs& A, unsigned f, int grid, int block, cudaStream_t s)
 {
-    switch (f & 7u) {
-    case 0: return launch_batch_one<R, 0>(B, grid, block, s);
-    case 1: return launch_batch_one<R, 1>(B, grid, block, s);
-    case 2: return launch_batch_one<R, 2>(B, grid, block, s);
-    case 3: return launch_batch_one<R, 3>(B, grid, block, s);
-    case 4: return launch_batch_one<R, 4>(B, grid, block, s);
-    case 5: return launch_batch_one<R, 5>(B, grid, block, s);
-    case 6: return launch_batch_one<R, 6>(B, grid, block, s);
-    default: return launch_batch_one<R, 7>(B, grid, block, s);
-    }
+    return with_features<split_rich<R, PH>()>(f, [&](auto F) { return launch_one<R, decltype(F)::value, PH>(A, grid, block, s); });
 }
 
 template <typename R, int PH>
 int occ_dispatch(unsigned f, int block)
 {
-    switch (f & 7u) {
-    case 0: return occupancy_one<R, 0, PH>(block);
-    case 1: return occupancy_one<R, 1, PH>(block);
-    case 2: return occupancy_one<R, 2, PH>(block);
-    case 3: return occupancy_one<R, 3, PH>(block);
-    case 4: return occupancy_one<R, 4, PH>(block);
-    case 5: return occupancy_one<R, 5, PH>(block);
-    case 6: return occupancy_one<R, 6, PH>(block);
-    default: return occupancy_one<R, 7, PH>(block);
-    }
+    return with_features<split_rich<R, PH>()>(f, [&](auto F) { return occupancy_one<R, decltype(F)::value, PH>(block); });
+}
+
+template <typename R>
+cudaError_t dispatch_batch(const BatchArgs& B, unsigned f, int grid, int block, cudaStream_t s)
+{
+    return with_features<false>(f, [&](auto F) { return launch_batch_one<R, decltype(F)::value>(B, grid, block, s); });
+}
+
+template <typename R>
+int batch_occ_dispatch(unsigned f, int block)
+{
+    return with_features<false>(f, [&](auto F) { return batch_occupancy_one<R, decltype(F)::value>(block); });
 }
 
 }  // namespace

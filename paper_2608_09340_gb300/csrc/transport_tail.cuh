@@ -22,11 +22,21 @@
 // packet continues bit for bit as it would have in a lane of its own.
 #pragma once
 
-// Warps of a CTA that walk packets this way, and packets per warp at the
-// start: beyond kTailWarps x kTailPerWarp running packets a CTA keeps to one
-// lane per packet, whose issue slots per event are a third of a group's.
+// Warps of a CTA that walk packets this way (their buffers take the stash's
+// place in shared memory). A CTA starts with up to kTailWide packets per warp
+// in groups of 8 lanes, or with nearly twice as many in groups of 4: these
+// use three times the issue slots per event of a lane's walk and gain less,
+// and a CTA with few packets above kTailWide rather waits for some to end.
+// Measured with both / with groups of 8 only / with groups of 4 from
+// 2 kTailWide down: outflow of 1e5 packets 399 / 415 / 399 ms, dusty slab
+// 113 / 124 / 113, the 1e4-packet slab (33 per CTA) 51 / 51 / 61.
 constexpr int kTailWarps = 8;
-constexpr int kTailPerWarp = 4;
+constexpr int kTailWide = 4;
+constexpr bool tail_starts(int total, int warps)
+{
+    return total <= warps * kTailWide || (total <= warps * 2 * kTailWide && 3 * total > warps * 4 * kTailWide);
+}
+
 // Rows inverted ahead (odd: no bank conflicts between slots). In the line's
 // core the frequency spreads by 0.7 and rows 0 to 6 (|x| < 2.67) hold nearly
 // all scatterings; a chain that leaves the window ends there and the window
@@ -149,7 +159,6 @@ __device__ __forceinline__ void shfl_packet(Pkt<float>& p, int src)
     p.rec.w = __shfl_sync(kFull, p.rec.w, src);
     p.nscat = __shfl_sync(kFull, p.nscat, src);
     p.ncross = __shfl_sync(kFull, p.ncross, src);
-    p.cell0 = __shfl_sync(kFull, p.cell0, src);
     p.id = __shfl_sync(kFull, p.id, src);
     p.vis_scat = __shfl_sync(kFull, p.vis_scat, src);
     if (F & F_RICH) {
@@ -166,7 +175,7 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
                           const Tabs& T, float a, float H0, LaneStats& st)
 {
     using O = Ops<float>;
-    constexpr bool VEL = (F & F_VEL) != 0, RICH = (F & F_RICH) != 0;
+    constexpr bool VEL = (F & F_VEL) != 0, RICH = (F & F_RICH) != 0, SEG = (F & F_SEG) != 0;
     const int lane = (int)(threadIdx.x & 31u);
     const bool absorbs = RICH && A.tau_abs;
     int sub = lane & (G - 1), base = lane - sub;
@@ -412,7 +421,7 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
         }
         if (VEL && ends) known = 0;
         // rich: the tallies of the segments that scattered, each by its lane
-        if (RICH && alive && (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)) && pos < now &&
+        if (SEG && alive && (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)) && pos < now &&
             (pos < f || (pos == f && ends && scat))) {
             float wseg = ow;
             if (absorbs) wseg = ow * fct;
@@ -460,7 +469,7 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
                 float wseg = p.wgt, fab = 0.0f;
                 if (absorbs) wseg = p.wgt * seg_factor<float>(__ldg(A.tau_abs + p.c) * s, fab);
                 if (A.rich & KRL_TALLY_EXC) p.vis_exc = fmaf(wseg * s, fH, p.vis_exc);
-                if (fk == 1 && lead && (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)))
+                if (SEG && fk == 1 && lead && (A.rich & (KRL_TALLY_J | KRL_TALLY_EMISS)))
                     rich_segment<float, F>(A, T, p.c, rec, p.nx, p.ny, p.nz, s, fc, fH, wseg);
                 if (absorbs) {
                     p.vis_abs = fmaf(p.wgt, fab, p.vis_abs);
