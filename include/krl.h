@@ -21,6 +21,11 @@
  *  - Caller buffers are BORROWED for the duration of the call only; the
  *    library copies what it keeps. The library owns everything it allocates
  *    and frees it in krl_grid_destroy.
+ *  - Device memory comes from two memory pools of the library's own per device
+ *    (grids and batches; scratch of a call). Of what they do not use they keep
+ *    at most 256 MiB and 6 GiB mapped across synchronisations; the scratch
+ *    pool is emptied with the device's last grid, and both before an
+ *    allocation is reported as failed.
  *  - Every call is ordered on the caller's stream `s` (a cudaStream_t; NULL
  *    is the legacy default stream). A call synchronises `s` only when it
  *    returns host data (documented per call).
@@ -265,7 +270,7 @@ typedef struct {
  * being captured into a CUDA graph keeps its slot inside the graph without
  * that wait: replays of such a graph must not overlap other runs of the grid.
  * An FP32 run of a line with an emissivity tally also allocates and frees
- * its segment buffer in stream order on `s` (cudaMallocAsync / cudaFreeAsync,
+ * its segment buffer in stream order on `s` (from the library's scratch pool,
  * size set by krl_tune.emiss_records), so the call stays capturable in a
  * CUDA graph; the buffer is the run's own and never outlives it.
  */
@@ -436,7 +441,7 @@ typedef struct {
  * alpha_k depends on the cell and the channel only, so it is tabulated once
  * per call in a stream-ordered scratch of ncell x n_ch floats, beside each
  * ray's starting cell and position (32 bytes per pixel, set up in FP64 once
- * per ray) (cudaMallocAsync on `s`, freed on `s` after the trace); with
+ * per ray) (from the library's scratch pool on `s`, freed on `s` after it); with
  * no_scratch, or when that memory is not available, the trace evaluates H per
  * segment and each ray's lanes set it up themselves, with the same result.
  */

@@ -24,6 +24,7 @@ struct krl_grid {
     double T_K = 0.0;
     int device = 0;
     int num_sms = 0;
+    bool counted = false;                // among its device's grids (device_pools)
     // owned copies of the fields
     float* opacity = nullptr;
     float* vel[3] = {nullptr, nullptr, nullptr};
@@ -102,43 +103,113 @@ krl_status cuda_fail(cudaError_t e, const char* what)
         if (e_ != cudaSuccess) return cuda_fail(e_, what); \
     } while (0)
 
+// Device memory comes from two stream-ordered pools of the library's own per
+// device, one for what grids and batches keep, one for the scratch of a call,
+// so that creating, replacing and destroying lines, and calls that the caller
+// waits for, do not map and unmap memory each time: a synchronisation unmaps
+// what a pool holds unused above its threshold, with the default pool all of
+// it (7 ms of a 27 ms ray trace with 4.3 GB of scratch). The thresholds bound
+// what stays mapped; with the device's last grid the scratch pool is emptied.
+struct DevicePools {
+    cudaMemPool_t kept = nullptr, scratch = nullptr;
+    int grids = 0;
+};
+constexpr unsigned long long kKeptIdle = 256ull << 20, kScratchIdle = 6ull << 30;
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+DevicePools g_pools[kMaxDevices];
+
+cudaError_t make_pool(int dev, unsigned long long idle, cudaMemPool_t* out)
+{
+    cudaMemPoolProps p{};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = dev;
+    cudaError_t e = cudaMemPoolCreate(out, &p);
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(*out, cudaMemPoolAttrReleaseThreshold, &idle);
+    return e;
+}
+
+// The current device's pools, made on first use. grids: change of its count
+// of grids.
+cudaError_t device_pools(DevicePools* out, int grids = 0)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    DevicePools& P = g_pools[dev];
+    if (!P.kept) e = make_pool(dev, kKeptIdle, &P.kept);
+    if (e == cudaSuccess && !P.scratch) e = make_pool(dev, kScratchIdle, &P.scratch);
+    P.grids += grids;
+    *out = P;
+    return e;
+}
+
+// From one of the pools, in the order of s; when there is no memory, once more
+// after unmapping what both hold unused.
+cudaError_t pool_alloc(void** p, size_t bytes, bool scratch, cudaStream_t s)
+{
+    DevicePools P;
+    cudaError_t e = device_pools(&P);
+    if (e != cudaSuccess) return e;
+    const cudaMemPool_t pool = scratch ? P.scratch : P.kept;
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        (void)cudaMemPoolTrimTo(P.kept, 0);
+        (void)cudaMemPoolTrimTo(P.scratch, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    }
+    return e;
+}
+
+// Kept memory: usable on every stream once s has been synchronised (each call
+// that allocates does so), and freed when nothing on the device uses it.
 template <typename T>
-cudaError_t dalloc(T** p, size_t n)
+cudaError_t dalloc(T** p, size_t n, cudaStream_t s)
 {
     *p = nullptr;
     if (n == 0) return cudaSuccess;
-    return cudaMalloc((void**)p, n * sizeof(T));
+    void* v = nullptr;
+    const cudaError_t e = pool_alloc(&v, n * sizeof(T), false, s);
+    if (e == cudaSuccess) *p = static_cast<T*>(v);
+    return e;
 }
 
 template <typename T>
-void dfree(T*& p)
+void dfree(T*& p, cudaStream_t s)
 {
-    if (p) cudaFree((void*)p);
+    if (p) cudaFreeAsync((void*)p, s);
     p = nullptr;
 }
 
-void free_line(krl_grid* g)
+// Frees the line's buffers in the order of s. Runs on other streams may still
+// use them: waits for the device first.
+void free_line(krl_grid* g, cudaStream_t s)
 {
-    dfree(g->cells);
-    dfree(g->eps);
-    dfree(g->src_rate);
-    dfree(g->src_cdf);
-    dfree(g->src_guide);
-    dfree(g->tab.voigt_lnH);
-    dfree(g->tab.H0);
-    dfree(g->tab.us_x);
-    dfree(g->tab.us_lncdf);
-    dfree(g->tab.us_guide);
-    dfree(g->tab.rtab);
-    dfree(g->tab.rquad);
-    dfree(g->tab.work);
-    dfree(g->spec_w);
-    dfree(g->spec_c);
-    dfree(g->scat);
-    dfree(g->exc);
-    dfree(g->J);
-    dfree(g->emiss);
-    dfree(g->scan_work);
+    if (g->cells) cudaDeviceSynchronize();
+    dfree(g->cells, s);
+    dfree(g->eps, s);
+    dfree(g->src_rate, s);
+    dfree(g->src_cdf, s);
+    dfree(g->src_guide, s);
+    dfree(g->tab.voigt_lnH, s);
+    dfree(g->tab.H0, s);
+    dfree(g->tab.us_x, s);
+    dfree(g->tab.us_lncdf, s);
+    dfree(g->tab.us_guide, s);
+    dfree(g->tab.rtab, s);
+    dfree(g->tab.rquad, s);
+    dfree(g->tab.work, s);
+    dfree(g->spec_w, s);
+    dfree(g->spec_c, s);
+    dfree(g->scat, s);
+    dfree(g->exc, s);
+    dfree(g->J, s);
+    dfree(g->emiss, s);
+    dfree(g->scan_work, s);
     g->line_ok = false;
 }
 
@@ -393,18 +464,21 @@ krl_status krl_grid_create(krl_grid** out, const krl_grid_desc* d, krl_stream st
     cudaGetDevice(&g->device);
     cudaDeviceGetAttribute(&g->num_sms, cudaDevAttrMultiProcessorCount, g->device);
     size_t n = (size_t)nc;
-    cudaError_t e = dalloc(&g->opacity, n);
+    DevicePools P;
+    cudaError_t e = device_pools(&P, 1);
+    g->counted = true;
+    if (e == cudaSuccess) e = dalloc(&g->opacity, n, s);
     const float* src[3] = {d->vx, d->vy, d->vz};
     g->has_vel = d->vx || d->vy || d->vz;
     for (int k = 0; k < 3 && e == cudaSuccess; ++k)
-        if (src[k]) e = dalloc(&g->vel[k], n);
-    if (e == cudaSuccess && d->n_coll) e = dalloc(&g->n_coll, n);
-    if (e == cudaSuccess && d->tau_abs) e = dalloc(&g->tau_abs, n);
-    if (e == cudaSuccess && d->tau_abs) e = dalloc(&g->absw, n);
-    if (e == cudaSuccess) e = dalloc(&g->stats, ST_N);
-    if (e == cudaSuccess) e = dalloc(&g->run_stats, (size_t)kSlots * ST_N);
-    if (e == cudaSuccess) e = dalloc(&g->next, (size_t)kSlots);
-    if (e == cudaSuccess) e = dalloc(&g->bad, 1);
+        if (src[k]) e = dalloc(&g->vel[k], n, s);
+    if (e == cudaSuccess && d->n_coll) e = dalloc(&g->n_coll, n, s);
+    if (e == cudaSuccess && d->tau_abs) e = dalloc(&g->tau_abs, n, s);
+    if (e == cudaSuccess && d->tau_abs) e = dalloc(&g->absw, n, s);
+    if (e == cudaSuccess) e = dalloc(&g->stats, ST_N, s);
+    if (e == cudaSuccess) e = dalloc(&g->run_stats, (size_t)kSlots * ST_N, s);
+    if (e == cudaSuccess) e = dalloc(&g->next, (size_t)kSlots, s);
+    if (e == cudaSuccess) e = dalloc(&g->bad, 1, s);
     for (int k = 0; k < kSlots && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&g->slot_ev[k], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemsetAsync(g->bad, 0, sizeof(int), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(g->opacity, d->opacity, n * 4, cudaMemcpyDeviceToDevice, s);
@@ -438,25 +512,36 @@ krl_status krl_grid_create(krl_grid** out, const krl_grid_desc* d, krl_stream st
 krl_status krl_grid_destroy(krl_grid* g)
 {
     if (!g) return KRL_OK;
+    int dev = g->device;
+    cudaGetDevice(&dev);
+    if (dev != g->device) cudaSetDevice(g->device);
     cudaDeviceSynchronize();
-    free_line(g);
-    dfree(g->opacity);
-    for (int k = 0; k < 3; ++k) dfree(g->vel[k]);
-    dfree(g->n_coll);
-    dfree(g->tau_abs);
-    dfree(g->absw);
-    dfree(g->lv_gamma);
-    dfree(g->lv_pops0);
-    dfree(g->lv_rate);
-    dfree(g->lv_total);
-    dfree(g->lv_change);
-    dfree(g->voigt2d);
-    dfree(g->stats);
-    dfree(g->run_stats);
-    dfree(g->next);
-    dfree(g->bad);
+    const cudaStream_t s = nullptr;             // (nothing is left to order against)
+    free_line(g, s);
+    dfree(g->opacity, s);
+    for (int k = 0; k < 3; ++k) dfree(g->vel[k], s);
+    dfree(g->n_coll, s);
+    dfree(g->tau_abs, s);
+    dfree(g->absw, s);
+    dfree(g->lv_gamma, s);
+    dfree(g->lv_pops0, s);
+    dfree(g->lv_rate, s);
+    dfree(g->lv_total, s);
+    dfree(g->lv_change, s);
+    dfree(g->voigt2d, s);
+    dfree(g->stats, s);
+    dfree(g->run_stats, s);
+    dfree(g->next, s);
+    dfree(g->bad, s);
     for (int k = 0; k < kSlots; ++k)
         if (g->slot_ev[k]) cudaEventDestroy(g->slot_ev[k]);
+    DevicePools P;
+    if (g->counted && device_pools(&P, -1) == cudaSuccess && P.grids == 0) {
+        cudaStreamSynchronize(s);
+        (void)cudaMemPoolTrimTo(P.scratch, 0);
+        (void)cudaMemPoolTrimTo(P.kept, kKeptIdle);
+    }
+    if (dev != g->device) cudaSetDevice(dev);
     delete g;
     return KRL_OK;
 }
@@ -487,7 +572,7 @@ krl_status krl_line_set(krl_grid* g, const krl_line_desc* d, krl_stream st)
     if ((d->tally_flags & KRL_TALLY_EMISS) && (d->n_cam < 1 || d->n_cam > KRL_MAX_CAMERAS))
         return fail(KRL_ERR_ARG, "emissivity needs 1..%d cameras", KRL_MAX_CAMERAS);
 
-    free_line(g);
+    free_line(g, s);
     KRL_CUDA(cudaMemsetAsync(g->bad, 0, sizeof(int), s), "krl_line_set");
     krl_line_desc L = *d;
     // keep a channel grid for the ray trace even without J / emissivity tallies
@@ -506,7 +591,7 @@ krl_status krl_line_set(krl_grid* g, const krl_line_desc* d, krl_stream st)
     g->info = I;
     if (L.ph_mode == 1) {
         if (!(I.a >= pow(10.0, kV2LaMin) && I.a <= pow(10.0, kV2LaMax))) {
-            free_line(g);
+            free_line(g, s);
             return fail(KRL_ERR_ARG, "ph_mode 1 needs 1e-6 <= a <= 1 (a = %g)", I.a);
         }
         const double s2 = (log10(I.a) - kV2LaMin) * ((kV2Na - 1) / (kV2LaMax - kV2LaMin));
@@ -516,7 +601,7 @@ krl_status krl_line_set(krl_grid* g, const krl_line_desc* d, krl_stream st)
         g->v2_w = s2 - j;
     } else if (L.ph_mode == 3) {
         if (!blend_crossing(I.a, &g->u0)) {
-            free_line(g);
+            free_line(g, s);
             return fail(KRL_ERR_ARG, "ph_mode 3: core and wing do not cross at a = %g", I.a);
         }
     }
@@ -524,32 +609,32 @@ krl_status krl_line_set(krl_grid* g, const krl_line_desc* d, krl_stream st)
     const size_t n = (size_t)g->ncell;
     const bool with_r = (L.tally_flags & KRL_TALLY_EMISS) != 0;
     const bool with_eps = L.k_ul > 0 && g->n_coll;
-    cudaError_t e = dalloc(&g->cells, n);
-    if (e == cudaSuccess && with_eps) e = dalloc(&g->eps, n);
-    if (e == cudaSuccess) e = dalloc(&g->tab.voigt_lnH, (size_t)kVoigtN);
-    if (e == cudaSuccess) e = dalloc(&g->tab.H0, 1);
-    if (e == cudaSuccess) e = dalloc(&g->tab.us_x, (size_t)kUsNx);
-    if (e == cudaSuccess) e = dalloc(&g->tab.us_lncdf, (size_t)kUsNx * kUsNu);
-    if (e == cudaSuccess) e = dalloc(&g->tab.us_guide, (size_t)kUsNx * kGuideN);
-    if (e == cudaSuccess && with_r) e = dalloc(&g->tab.rtab, kRtabElems);
-    if (e == cudaSuccess && with_r) e = dalloc(&g->tab.rquad, kRquadElems);
-    if (e == cudaSuccess) e = dalloc(&g->tab.work, line_tables_work_doubles());
-    if (e == cudaSuccess) e = dalloc(&g->spec_w, (size_t)L.spec_nbins + 2);
-    if (e == cudaSuccess) e = dalloc(&g->spec_c, (size_t)L.spec_nbins + 2);
-    if (e == cudaSuccess && (L.tally_flags & KRL_TALLY_SCATMAP)) e = dalloc(&g->scat, n);
-    if (e == cudaSuccess && (L.tally_flags & KRL_TALLY_EXC)) e = dalloc(&g->exc, n);
-    if (e == cudaSuccess && (L.tally_flags & KRL_TALLY_J)) e = dalloc(&g->J, n * L.n_ch);
-    if (e == cudaSuccess && with_r) e = dalloc(&g->emiss, (size_t)L.n_cam * n * L.n_ch);
+    cudaError_t e = dalloc(&g->cells, n, s);
+    if (e == cudaSuccess && with_eps) e = dalloc(&g->eps, n, s);
+    if (e == cudaSuccess) e = dalloc(&g->tab.voigt_lnH, (size_t)kVoigtN, s);
+    if (e == cudaSuccess) e = dalloc(&g->tab.H0, 1, s);
+    if (e == cudaSuccess) e = dalloc(&g->tab.us_x, (size_t)kUsNx, s);
+    if (e == cudaSuccess) e = dalloc(&g->tab.us_lncdf, (size_t)kUsNx * kUsNu, s);
+    if (e == cudaSuccess) e = dalloc(&g->tab.us_guide, (size_t)kUsNx * kGuideN, s);
+    if (e == cudaSuccess && with_r) e = dalloc(&g->tab.rtab, kRtabElems, s);
+    if (e == cudaSuccess && with_r) e = dalloc(&g->tab.rquad, kRquadElems, s);
+    if (e == cudaSuccess) e = dalloc(&g->tab.work, line_tables_work_doubles(), s);
+    if (e == cudaSuccess) e = dalloc(&g->spec_w, (size_t)L.spec_nbins + 2, s);
+    if (e == cudaSuccess) e = dalloc(&g->spec_c, (size_t)L.spec_nbins + 2, s);
+    if (e == cudaSuccess && (L.tally_flags & KRL_TALLY_SCATMAP)) e = dalloc(&g->scat, n, s);
+    if (e == cudaSuccess && (L.tally_flags & KRL_TALLY_EXC)) e = dalloc(&g->exc, n, s);
+    if (e == cudaSuccess && (L.tally_flags & KRL_TALLY_J)) e = dalloc(&g->J, n * L.n_ch, s);
+    if (e == cudaSuccess && with_r) e = dalloc(&g->emiss, (size_t)L.n_cam * n * L.n_ch, s);
     if (e == cudaSuccess && L.src_kind == KRL_SRC_VOLUME) {
-        e = dalloc(&g->src_rate, n);
-        if (e == cudaSuccess) e = dalloc(&g->src_cdf, n);
-        if (e == cudaSuccess) e = dalloc(&g->src_guide, ((size_t)1 << kCdfGuideBits) + 1);
+        e = dalloc(&g->src_rate, n, s);
+        if (e == cudaSuccess) e = dalloc(&g->src_cdf, n, s);
+        if (e == cudaSuccess) e = dalloc(&g->src_guide, ((size_t)1 << kCdfGuideBits) + 1, s);
         g->scan_work_n = emission_cdf_work_doubles(g->ncell);
-        if (e == cudaSuccess) e = dalloc(&g->scan_work, g->scan_work_n);
+        if (e == cudaSuccess) e = dalloc(&g->scan_work, g->scan_work_n, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(g->src_rate, L.src_rate, n * 4, cudaMemcpyDeviceToDevice, s);
     }
     if (e != cudaSuccess) {
-        free_line(g);
+        free_line(g, s);
         return cuda_fail(e, "krl_line_set allocation");
     }
     g->has_rtab = with_r;
@@ -572,31 +657,32 @@ krl_status krl_line_set(krl_grid* g, const krl_line_desc* d, krl_stream st)
     e = derive_fields(F, s);
     if (e == cudaSuccess) e = build_line_tables(I.a, g->tab, with_r, s);
     if (e == cudaSuccess && L.ph_mode == 1 && !g->voigt2d) {
-        e = dalloc(&g->voigt2d, (size_t)kV2Na * kV2Nx);
+        e = dalloc(&g->voigt2d, (size_t)kV2Na * kV2Nx, s);
         if (e == cudaSuccess) e = build_voigt2d(g->voigt2d, g->tab.work, s);
     }
     if (e == cudaSuccess && L.src_kind == KRL_SRC_VOLUME)
         e = emission_cdf(g->src_rate, g->ncell, g->src_cdf, g->scan_work, g->scan_work_n, g->bad, s);
     if (e == cudaSuccess && L.src_kind == KRL_SRC_VOLUME) e = emission_guide(g->src_cdf, g->ncell, g->src_guide, s);
     if (e != cudaSuccess) {
-        free_line(g);
+        free_line(g, s);
         return cuda_fail(e, "krl_line_set kernels");
     }
     krl_status zs = zero_tallies(g, s);
     if (zs != KRL_OK) return zs;
-    // H(a, 0) for krl_line_info_get (small synchronous copy on this stream)
+    // H(a, 0) for krl_line_info_get and the source check (small copies on this
+    // stream; the synchronisation also makes the new buffers safe on others)
     float h0 = 0.0f;
+    int bad = 0;
     e = cudaMemcpyAsync(&h0, g->tab.H0, sizeof(float), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, g->bad, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "krl_line_set");
-    int bad = 0;
-    cudaMemcpy(&bad, g->bad, sizeof(int), cudaMemcpyDeviceToHost);
     if (bad & 2) {
-        free_line(g);
+        free_line(g, s);
         return fail(KRL_ERR_ARG, "volume source rate sums to zero");
     }
     if (bad) {
-        free_line(g);
+        free_line(g, s);
         return fail(KRL_ERR_NUMERIC, "volume source rate holds NaN/Inf or a negative value");
     }
     g->info.H0 = h0;
@@ -678,7 +764,7 @@ krl_status krl_run_packets(krl_grid* g, uint64_t n, uint64_t first_id, uint64_t 
         const unsigned long long lo = 1ull << 16, hi = 1ull << 25;
         unsigned long long cap = (unsigned long long)T.emiss_records;
         if (cap == 0) cap = n > hi / 64 ? hi : (n * 64 < lo ? lo : n * 64);
-        if (cudaMallocAsync(&segbuf, 16 + (size_t)cap * 32, s) == cudaSuccess) {
+        if (pool_alloc(&segbuf, 16 + (size_t)cap * 32, true, s) == cudaSuccess) {
             A.seg_count = static_cast<unsigned long long*>(segbuf);
             A.seg = reinterpret_cast<float4*>(static_cast<char*>(segbuf) + 16);
             A.seg_cap = cap;
@@ -802,7 +888,7 @@ krl_status krl_raytrace_channels(krl_grid* g, const krl_raytrace_desc* d, float*
     const size_t rbytes = (size_t)d->npix_x * (size_t)d->npix_y * 2 * sizeof(float4);
     A.hcube = nullptr;
     A.rayinit = nullptr;
-    if (!d->no_scratch && cudaMallocAsync((void**)&A.hcube, hbytes + rbytes, s) != cudaSuccess) {
+    if (!d->no_scratch && pool_alloc((void**)&A.hcube, hbytes + rbytes, true, s) != cudaSuccess) {
         (void)cudaGetLastError();
         A.hcube = nullptr;
     }
@@ -837,18 +923,24 @@ extern "C" {
 krl_status krl_batch_destroy(krl_batch* b)
 {
     if (!b) return KRL_OK;
+    int dev = b->device;
+    cudaGetDevice(&dev);
+    if (dev != b->device) cudaSetDevice(b->device);
     cudaDeviceSynchronize();
+    const cudaStream_t s = nullptr;
     if (b->h_args) cudaFreeHost(b->h_args);
-    dfree(b->d_args);
-    dfree(b->d_counts);
-    dfree(b->d_dst);
-    dfree(b->d_cursor);
+    dfree(b->d_args, s);
+    dfree(b->d_counts, s);
+    dfree(b->d_dst, s);
+    dfree(b->d_cursor, s);
+    if (dev != b->device) cudaSetDevice(dev);
     delete b;
     return KRL_OK;
 }
 
 krl_status krl_batch_create(krl_batch** out, krl_grid* const* grids, int n_models, krl_stream st)
 {
+    cudaStream_t s = (cudaStream_t)st;
     if (!out || !grids || n_models < 1) return fail(KRL_ERR_ARG, "krl_batch_create: bad arguments");
     *out = nullptr;
     int dev = 0;
@@ -871,10 +963,10 @@ krl_status krl_batch_create(krl_batch** out, krl_grid* const* grids, int n_model
     }
     const size_t n = (size_t)n_models;
     cudaError_t e = cudaMallocHost((void**)&b->h_args, n * sizeof(TransportArgs));
-    if (e == cudaSuccess) e = dalloc(&b->d_args, n);
-    if (e == cudaSuccess) e = dalloc(&b->d_counts, n * (1 + ST_N));
-    if (e == cudaSuccess) e = dalloc(&b->d_dst, n);
-    if (e == cudaSuccess) e = dalloc(&b->d_cursor, 1);
+    if (e == cudaSuccess) e = dalloc(&b->d_args, n, s);
+    if (e == cudaSuccess) e = dalloc(&b->d_counts, n * (1 + ST_N), s);
+    if (e == cudaSuccess) e = dalloc(&b->d_dst, n, s);
+    if (e == cudaSuccess) e = dalloc(&b->d_cursor, 1, s);
     if (e == cudaSuccess) {
         std::vector<unsigned long long*> dst(n);
         for (size_t m = 0; m < n; ++m) dst[m] = grids[m]->stats;
@@ -988,15 +1080,17 @@ krl_status level_const(const krl_grid* g, const krl_levels_desc* d, LevelConst& 
     return KRL_OK;
 }
 
-krl_status level_scratch(krl_grid* g)
+krl_status level_scratch(krl_grid* g, cudaStream_t s)
 {
     const size_t n = (size_t)g->ncell;
+    if (g->lv_gamma && g->lv_pops0 && g->lv_rate && g->lv_total && g->lv_change) return KRL_OK;
     cudaError_t e = cudaSuccess;
-    if (!g->lv_gamma) e = dalloc(&g->lv_gamma, (size_t)kMaxTrans * n);
-    if (e == cudaSuccess && !g->lv_pops0) e = dalloc(&g->lv_pops0, (size_t)kMaxLevels * n);
-    if (e == cudaSuccess && !g->lv_rate) e = dalloc(&g->lv_rate, n);
-    if (e == cudaSuccess && !g->lv_total) e = dalloc(&g->lv_total, levels_sum_scratch_doubles());
-    if (e == cudaSuccess && !g->lv_change) e = dalloc(&g->lv_change, 1);
+    if (!g->lv_gamma) e = dalloc(&g->lv_gamma, (size_t)kMaxTrans * n, s);
+    if (e == cudaSuccess && !g->lv_pops0) e = dalloc(&g->lv_pops0, (size_t)kMaxLevels * n, s);
+    if (e == cudaSuccess && !g->lv_rate) e = dalloc(&g->lv_rate, n, s);
+    if (e == cudaSuccess && !g->lv_total) e = dalloc(&g->lv_total, levels_sum_scratch_doubles(), s);
+    if (e == cudaSuccess && !g->lv_change) e = dalloc(&g->lv_change, 1, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);     // a later call may come on another stream
     if (e != cudaSuccess) return cuda_fail(e, "level scratch");
     return KRL_OK;
 }
@@ -1014,7 +1108,7 @@ krl_status krl_levels_solve(krl_grid* g, const krl_levels_desc* d, const double*
     krl_status ls = level_const(g, d, L);
     if (ls != KRL_OK) return ls;
     if (L.n_trans > 0 && !gamma) return fail(KRL_ERR_ARG, "gamma is required when the levels have lines");
-    ls = level_scratch(g);
+    ls = level_scratch(g, s);
     if (ls != KRL_OK) return ls;
     KRL_CUDA(cudaMemsetAsync(g->lv_change, 0, sizeof(unsigned long long), s), "levels");
     KRL_CUDA(levels_solve(L, gamma, g->ncell, g->n_coll, d->n_mol, pops, g->lv_change, s), "levels solve");
@@ -1037,7 +1131,7 @@ krl_status krl_levels_iterate(krl_grid* g, const krl_levels_desc* d, int n_iter,
     LevelConst L;
     krl_status ls = level_const(g, d, L);
     if (ls != KRL_OK) return ls;
-    ls = level_scratch(g);
+    ls = level_scratch(g, s);
     if (ls != KRL_OK) return ls;
     const int ncell = g->ncell;
     const size_t n = (size_t)ncell;
