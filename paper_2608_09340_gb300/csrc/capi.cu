@@ -721,16 +721,23 @@ krl_status krl_run_packets(krl_grid* g, uint64_t n, uint64_t first_id, uint64_t 
             return fail(KRL_ERR_ARG, "table_space = constant needs ph_mode 2 and the FP32 walk");
         mode = 4;
     }
-    // The rich walk without per-segment tallies has a form with more warps per
-    // SM, which pays when packets outnumber the lanes of the general form (two
-    // 256-thread CTAs per SM) twice; with fewer, a launch is its longest
-    // packets, and they run faster among fewer warps. Dusty slab of tau0 = 1e4,
-    // 1e5 / 2e5 / 8e5 packets on 77824 lanes: 116 / 145 / 351 ms against 101 /
-    // 154 / 388.
-    if ((f & F_RICH) && !(f & F_SEG) && mode == 2 && T.precision == KRL_PREC_FP32 && !T.block &&
-        n >= 2ull * 2ull * 256ull * (unsigned)g->num_sms) {
-        T.block = transport_light_block();
-        f |= F_WIDE;
+    // The production walk without per-segment tallies has a form with more
+    // warps per SM, which pays when packets outnumber the lanes of the other
+    // one (two 256-thread CTAs per SM) twice; with fewer, a launch is set by
+    // its longest packets, and they run faster among fewer warps with more
+    // registers. Dusty slab of tau0 = 1e4, 1e5 / 2e5 / 8e5 packets on 77824
+    // lanes, wide against narrow: 116 / 145 / 351 ms against 101 / 154 / 388;
+    // Table 1 box, 1e5 / 3e5 / 1e6 packets: 9.3 / 13.9 / 27.7 against 9.1 /
+    // 14.4 / 32.2.
+    if (!(f & F_SEG) && mode == 2 && T.precision == KRL_PREC_FP32) {
+        if (T.block) {
+            if (!(f & F_RICH)) f |= F_WIDE;     // the lean walk takes any CTA up to 512
+        } else if (n >= 2ull * 2ull * 256ull * (unsigned)g->num_sms) {
+            f |= F_WIDE;
+            T.block = transport_wide_block(f);
+        } else {
+            T.block = 256;
+        }
     }
     if (!T.block) T.block = maxb;
     int occ = transport_occupancy(T.precision, f, T.block, mode);

@@ -65,7 +65,7 @@ enum : unsigned {
     F_SCAT = 2u,      // per-cell scattering counts
     F_RICH = 4u,      // any of excitation, mean intensity, emissivity, destruction, continuum
     F_SEG = 8u,       // (with F_RICH) mean intensity or emissivity: tallies of every segment
-    F_WIDE = 16u,     // (with F_RICH, without F_SEG) in the larger CTA, transport_light_block()
+    F_WIDE = 16u,     // (not with F_SEG) in the larger CTA, transport_wide_block()
 };
 
 enum { ST_EMITTED = 0, ST_ESCAPED, ST_DESTROYED, ST_STUCK, ST_SCAT, ST_CROSS, ST_ABSORBED, ST_N = 8 };
@@ -201,7 +201,7 @@ int transport_occupancy_ph(int ph_mode, int precision, unsigned features, int bl
 // Largest CTA the instantiation is compiled for (512 lean FP32, else 256).
 int transport_max_block(int precision, unsigned features);
 // CTA of the F_WIDE walk (FP32, profile mode 2).
-int transport_light_block();
+int transport_wide_block(unsigned features);
 // The batched launch: its CTA size limit and occupancy.
 int transport_batch_max_block();
 int transport_batch_occupancy(int precision, unsigned features, int block);

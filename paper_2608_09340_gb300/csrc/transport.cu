@@ -45,7 +45,7 @@ int transport_max_block(int precision, unsigned features)
     return (precision == KRL_PREC_FP32 && !(features & F_RICH)) ? 512 : 256;
 }
 
-int transport_light_block() { return kLightBlock; }
+int transport_wide_block(unsigned features) { return features & F_RICH ? kLightBlock : kLeanBlock; }
 
 int transport_occupancy(int precision, unsigned features, int block, int ph_mode)
 {

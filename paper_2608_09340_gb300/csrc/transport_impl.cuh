@@ -1057,18 +1057,20 @@ __device__ __forceinline__ T warp_sum(T v)
     return v;
 }
 
-// Launch shape per instantiation, two CTAs per SM each: the lean FP32 walk
-// runs 512-thread CTAs (64 registers each), the FP32 walk with weights,
-// destruction or excitation but no per-segment tallies 384 (F_WIDE, 80
-// registers) or 256, the others, which need more registers, 256. Shared memory holds two CTAs'
-// tables, so more warps per SM mean larger CTAs. On the 128^3 cloud (86 events
-// per packet, 16 warps per SM issued in half the cycles) 384 threads took the
-// Lambda cycle from 79 to 66 ms, 512 (with spills) 75.
-constexpr int kLightBlock = 384;
+// Launch shape per instantiation, two CTAs per SM each (shared memory holds
+// two CTAs' tables). F_WIDE: the lean FP32 walk in 512-thread CTAs (64
+// registers each) and the rich one without per-segment tallies in 384 (80
+// registers), for throughput; all others, and these two where a launch is set
+// by its longest packets, in 256 (up to 128 registers, which the walk of the
+// last packets uses: a step of its frequency chain takes 136 cycles, 173 with
+// 64 registers). On the 128^3 cloud (86 events per packet; 16 warps per SM
+// issued in half the cycles) 384 threads took the Lambda cycle from 79 to
+// 66 ms, 512 (with spills) 75.
+constexpr int kLeanBlock = 512, kLightBlock = 384;
 template <typename R, unsigned F>
 constexpr int max_block()
 {
-    return sizeof(R) == 8 || (F & F_RICH) ? ((F & F_WIDE) ? kLightBlock : 256) : 512;
+    return sizeof(R) == 8 || !(F & F_WIDE) ? 256 : ((F & F_RICH) ? kLightBlock : kLeanBlock);
 }
 
 // ---------------------------------------------------------------- tail compaction
@@ -1788,52 +1790,56 @@ int batch_occupancy_one(int block)
     return n;
 }
 
-// Calls fn with the instantiation of the features f. The walk without
-// per-segment tallies has instantiations of its own in the FP32 production
-// walk only (SPLIT); elsewhere the rich walk handles all of them.
+// Calls fn with the instantiation of the features f. The narrow lean walk and
+// the rich walk without per-segment tallies have instantiations of their own
+// in the FP32 production walk only (SPLIT).
 template <bool SPLIT, typename Fn>
 auto with_features(unsigned f, Fn fn)
 {
     using std::integral_constant;
+    constexpr unsigned W = F_WIDE, L = F_RICH, S = F_RICH | F_SEG;
     if constexpr (SPLIT) {
-        constexpr unsigned W = F_RICH | F_WIDE;
         switch (f & (F_RICH | F_SEG | F_WIDE | 3u)) {
-        case F_RICH: return fn(integral_constant<unsigned, F_RICH>());
-        case F_RICH | 1u: return fn(integral_constant<unsigned, F_RICH | 1u>());
-        case F_RICH | 2u: return fn(integral_constant<unsigned, F_RICH | 2u>());
-        case F_RICH | 3u: return fn(integral_constant<unsigned, F_RICH | 3u>());
-        case W: return fn(integral_constant<unsigned, W>());
-        case W | 1u: return fn(integral_constant<unsigned, W | 1u>());
-        case W | 2u: return fn(integral_constant<unsigned, W | 2u>());
-        case W | 3u: return fn(integral_constant<unsigned, W | 3u>());
+        case 0: return fn(integral_constant<unsigned, 0u>());
+        case 1: return fn(integral_constant<unsigned, 1u>());
+        case 2: return fn(integral_constant<unsigned, 2u>());
+        case 3: return fn(integral_constant<unsigned, 3u>());
+        case L: return fn(integral_constant<unsigned, L>());
+        case L | 1u: return fn(integral_constant<unsigned, L | 1u>());
+        case L | 2u: return fn(integral_constant<unsigned, L | 2u>());
+        case L | 3u: return fn(integral_constant<unsigned, L | 3u>());
+        case L | W: return fn(integral_constant<unsigned, L | W>());
+        case L | W | 1u: return fn(integral_constant<unsigned, L | W | 1u>());
+        case L | W | 2u: return fn(integral_constant<unsigned, L | W | 2u>());
+        case L | W | 3u: return fn(integral_constant<unsigned, L | W | 3u>());
         default: break;
         }
     }
     switch (f & 7u) {
-    case 0: return fn(integral_constant<unsigned, 0u>());
-    case 1: return fn(integral_constant<unsigned, 1u>());
-    case 2: return fn(integral_constant<unsigned, 2u>());
-    case 3: return fn(integral_constant<unsigned, 3u>());
-    case 4: return fn(integral_constant<unsigned, F_RICH | F_SEG>());
-    case 5: return fn(integral_constant<unsigned, F_RICH | F_SEG | 1u>());
-    case 6: return fn(integral_constant<unsigned, F_RICH | F_SEG | 2u>());
-    default: return fn(integral_constant<unsigned, F_RICH | F_SEG | 3u>());
+    case 0: return fn(integral_constant<unsigned, W>());
+    case 1: return fn(integral_constant<unsigned, W | 1u>());
+    case 2: return fn(integral_constant<unsigned, W | 2u>());
+    case 3: return fn(integral_constant<unsigned, W | 3u>());
+    case 4: return fn(integral_constant<unsigned, S>());
+    case 5: return fn(integral_constant<unsigned, S | 1u>());
+    case 6: return fn(integral_constant<unsigned, S | 2u>());
+    default: return fn(integral_constant<unsigned, S | 3u>());
     }
 }
 
 template <typename R, int PH>
-constexpr bool split_rich() { return sizeof(R) == 4 && PH == 2; }
+constexpr bool split() { return sizeof(R) == 4 && PH == 2; }
 
 template <typename R, int PH>
 cudaError_t dispatch(const TransportArgs& A, unsigned f, int grid, int block, cudaStream_t s)
 {
-    return with_features<split_rich<R, PH>()>(f, [&](auto F) { return launch_one<R, decltype(F)::value, PH>(A, grid, block, s); });
+    return with_features<split<R, PH>()>(f, [&](auto F) { return launch_one<R, decltype(F)::value, PH>(A, grid, block, s); });
 }
 
 template <typename R, int PH>
 int occ_dispatch(unsigned f, int block)
 {
-    return with_features<split_rich<R, PH>()>(f, [&](auto F) { return occupancy_one<R, decltype(F)::value, PH>(block); });
+    return with_features<split<R, PH>()>(f, [&](auto F) { return occupancy_one<R, decltype(F)::value, PH>(block); });
 }
 
 template <typename R>

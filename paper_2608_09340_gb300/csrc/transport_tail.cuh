@@ -46,8 +46,7 @@ constexpr int kUWin = 7;
 // A warp's buffers. Slots are lanes; the arrays of the two serial loops are in
 // chain order (index: first lane of the group + place in the chain), so that
 // the loops read at constant offsets. They run in fours and may read past
-// their group's part, whose values are then not used (an offset read there is
-// a slot's, or the zero that d holds).
+// their group's part, whose values are then not used.
 struct TailBuf {
     float4 a[32];               // {z1, sin(gamma), g - 1, byte offset of the slot's row 0 in u}
     float2 b[32];               // {first row of u, z2}
@@ -59,8 +58,9 @@ struct TailBuf {
             float xs[68];       // [2 x first lane + k]: lab-frame frequency in front of scattering k
         };
         struct {
-            float4 c[32];       // {ds, n_in}
-            float4 d[32];       // rich: {absorbed fraction, mean-weight factor, H, -}
+            float4 d[32];       // rich: {absorbed fraction, mean-weight factor, H, 0}
+            float2 c[3][32];    // {ds, n_in's component}
+            float o[3][32];     // position in front of the segment, by component
         };
     };
 };
@@ -187,7 +187,6 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
     bool out = false, far = false;              // its row lies outside its window; |x| > 300
     float mx = 0.0f, my = 0.0f, mz = 0.0f, tn = 0.0f, ueps = 1.0f;
     tb->a[lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // (offset 0: every slot's window lies in u from here on)
-    tb->ac[lane] = tb->ac[lane + 32] = tb->a[lane];
     tb->b[lane] = make_float2(0.0f, 0.0f);
     int len = 16;               // about the run of scatterings between two crossings
     for (;;) {
@@ -278,7 +277,11 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
         float x = (known ? xe : p.x) + 0.0f;
         const float xb = x, vb = VEL ? vdot<float>(p.nx, p.ny, p.nz, p.rec) : 0.0f;
         float vd = vb;
+        // (both halves of ac: a group with known scatterings reads past its part
+        // into the next one's or the upper half, and every offset there has to
+        // be a slot's)
         tb->ac[base + pos] = tb->a[lane];
+        tb->ac[32 + lane] = tb->a[lane];
         if (VEL) tb->vc[base + pos] = vdot<float>(mx, my, mz, p.rec);
         __syncwarp();
         const float4* pa = tb->ac + (base + known);
@@ -347,7 +350,9 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
         }
         const float alpha = __fmul_rn(p.rec.x, H);
         const float ds = O::dv(ti, alpha);
-        tb->c[base + pos] = make_float4(ds, ix, iy, iz);
+        tb->c[0][base + pos] = make_float2(ds, ix);
+        tb->c[1][base + pos] = make_float2(ds, iy);
+        tb->c[2][base + pos] = make_float2(ds, iz);
         float ab = 0.0f, fct = 1.0f;
         if (RICH) {
             if (absorbs) fct = seg_factor<float>(__ldg(A.tau_abs + p.c) * ds, ab);
@@ -355,26 +360,26 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
         }
         __syncwarp();
 
-        // ---- positions (and, rich, weights and visit sums) in front of each segment
-        float2 qxy = make_float2(p.px, p.py), oxy = qxy;
-        float qz = p.pz, oz = qz;
+        // ---- positions (and, rich, weights and visit sums) in front of each
+        // segment: a lane follows one component, which leaves a step one read,
+        // one write and one fused multiply-add
+        const int comp = (sub & 3) < 3 ? sub & 3 : 2;
+        float qc = comp == 0 ? p.px : (comp == 1 ? p.py : p.pz);
         float w = p.wgt, ve = p.vis_exc, va = p.vis_abs, ow = w, oe = ve, oa = va;
-        const float4* pc = tb->c + base;
+        const float2* pc = &tb->c[comp][base];
+        float* po = &tb->o[comp][base];
         const float4* pd = tb->d + base;
 #pragma unroll 1
-        for (int k0 = 0; k0 < now4; k0 += 4, pc += 4, pd += 4) {
-            float4 v[4];
+        for (int k0 = 0; k0 < now4; k0 += 4, pc += 4, po += 4, pd += 4) {
+            float2 v[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) v[q] = pc[q];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const bool mine = k0 + q == pos;
-                oxy.x = mine ? qxy.x : oxy.x;
-                oxy.y = mine ? qxy.y : oxy.y;
-                oz = mine ? qz : oz;
-                qxy = __ffma2_rn(make_float2(v[q].x, v[q].x), make_float2(v[q].y, v[q].z), qxy);
-                qz = fmaf(v[q].x, v[q].w, qz);
+                po[q] = qc;
+                qc = fmaf(v[q].x, v[q].y, qc);
                 if (RICH) {
+                    const bool mine = k0 + q == pos;
                     const float4 d = pd[q];
                     ow = mine ? w : ow;
                     oe = mine ? ve : oe;
@@ -383,6 +388,9 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
                 }
             }
         }
+        __syncwarp();
+        const float2 oxy = make_float2(tb->o[0][base + pos], tb->o[1][base + pos]);
+        const float oz = tb->o[2][base + pos];
         // ---- how many of the scatterings stand: up to the first segment that
         // leaves the cell or ends the packet, or whose row was not at hand,
         // and within the event budget
@@ -398,15 +406,17 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
         }
         // bit k: the chain's k-th segment
         unsigned stop = __ballot_sync(kFull, pos < now && (!scat || gone || dead)) >> base;
-        unsigned lost = __ballot_sync(kFull, pos < now && out) >> base;
-        unsigned past = __ballot_sync(kFull, pos < now && far) >> base;
         const unsigned group = G < 32 ? (1u << G) - 1u : kFull;
         auto order = [&](unsigned bits) {
             bits &= group;
             return ((bits >> s0) | (s0 ? bits << (G - s0) : 0u)) & group;
         };
         stop = order(stop);
-        lost = order(lost) | order(past) << 1;
+        unsigned lost = 0u;
+        if (__any_sync(kFull, pos < now && (out || far))) {     // rare
+            lost = order(__ballot_sync(kFull, pos < now && out) >> base);
+            lost |= order(__ballot_sync(kFull, pos < now && far) >> base) << 1;
+        }
         int lim = room < (uint32_t)now ? (int)room : now;
         const int fo = lost ? __ffs(lost) - 1 : 64;     // its profile and place are right, its outcome is not
         int f = stop ? __ffs(stop) - 1 : now;
