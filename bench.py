@@ -48,7 +48,7 @@ OPS_PER_CROSS = 32
 FP32_LANES_PER_SM = 128
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "transport_sphere64_tau1e4.txt")
 KERNEL_SRC = [os.path.join(ROOT, "paper_2608_09340_gb300", "csrc", f)
-              for f in ("transport_impl.cuh", "transport.cu", "krl_internal.cuh")]
+              for f in ("transport_impl.cuh", "transport_tail.cuh", "transport.cu", "krl_internal.cuh")]
 
 
 def parse():

@@ -199,8 +199,10 @@ typedef struct {
     int precision;              /* KRL_PREC_FP32 (production) or KRL_PREC_FP64
                                    (same walk in double, for lockstep checks)       */
     int block;                  /* threads per CTA, multiple of 32; at most 512 for
-                                   the FP32 walk without rich tallies (its default),
-                                   256 otherwise (the default there)               */
+                                   the FP32 walk without rich tallies, 256 otherwise.
+                                   0: 256, or 512 (384 with continuum or excitation
+                                   tallies) in FP32 runs of profile mode 2 without
+                                   per-segment tallies that have many packets      */
     int ctas_per_sm;            /* resident CTAs per SM of the persistent grid      */
     int refill_min;             /* a warp takes new packets once at least this many
                                    of its lanes are idle (1..32); 0: the walk
@@ -212,7 +214,7 @@ typedef struct {
     int64_t emiss_records;      /* FP32 runs with an emissivity tally deposit it in
                                    two stages: the walk records each segment (32 B)
                                    in a stream-ordered buffer of this many records,
-                                   then one warp per segment adds its channels.
+                                   then a second kernel adds their channels.
                                    0: 64 per packet, clamped to [2^16, 2^25];
                                    -1: deposit inside the walk (no buffer); at most
                                    2^36 (KRL_ERR_ARG beyond). Segments

@@ -392,7 +392,7 @@ constexpr int kTraceBlock = 128;
 // The values are those of the full formula in every lane. With one ray's 64
 // channels over 16 lanes (every warp has a line-centre lane) the trace of
 // 256^3 cells x 64 channels at 1024^2 pixels took 22.3 ms, bound by issue and
-// special-function slots.
+// special-function slots; in this layout 16.
 // The cube holds the extinction alpha0 H + alpha_abs (JL false) or H (JL true:
 // the line-emission term needs H; alpha is formed here).
 template <int CPL, int D, int MINB, bool JL, bool VEC>

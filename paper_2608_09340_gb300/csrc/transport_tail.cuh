@@ -10,13 +10,15 @@
 // scatterings of its packet, one per lane: each lane makes its scattering's
 // draws, the angle to the previous scattering's direction, and the sampler's
 // inversion at its ln(xi) in the kUWin rows around the packet's |x|. What
-// remains serial is the chain of frequencies, x -> row -> u_par -> x' (about
-// 150 cycles), walked for up to G scatterings on the assumption that all
-// happen in this cell. Then each lane evaluates the profile and the distance
+// remains serial is the chain of frequencies, x -> row -> u_par -> x' (136
+// cycles a step with 128 registers, 173 with 64), walked for up to G
+// scatterings on the assumption that all happen in this cell. Then each lane evaluates the profile and the distance
 // of its own segment, the positions follow as a chain of fused multiply-adds,
 // and the first lane whose point lies outside the cell (or that ends the
 // packet) marks how many of the scatterings stand; the rest are walked again
-// from the next cell, with the same draws.
+// from the next cell, with the same draws. A packet alone then takes 150 to
+// 200 ns per event (690 to 1000 before): 1e5 packets in the outflowing sphere
+// 938 -> 396 ms, 1e4 in the slab 138 -> 33 ms, together with the other steps.
 //
 // Every value is formed by the functions and in the order of advance(), so a
 // packet continues bit for bit as it would have in a lane of its own.
@@ -27,9 +29,10 @@
 // in groups of 8 lanes, or with nearly twice as many in groups of 4: these
 // use three times the issue slots per event of a lane's walk and gain less,
 // and a CTA with few packets above kTailWide rather waits for some to end.
-// Measured with both / with groups of 8 only / with groups of 4 from
-// 2 kTailWide down: outflow of 1e5 packets 399 / 415 / 399 ms, dusty slab
-// 113 / 124 / 113, the 1e4-packet slab (33 per CTA) 51 / 51 / 61.
+// Measured with both / with groups of 8 only, means of three seeds: outflow of
+// 1e5 packets 368 / 369 ms, static sphere 492 / 500, dusty slab 107 / 109,
+// 64 models 162 / 167, 1e4-packet slab 35.8 / 35.1; with groups of 4 from
+// 2 kTailWide down the slab (33 packets per CTA) took 52 for 44.
 constexpr int kTailWarps = 8;
 constexpr int kTailWide = 4;
 constexpr bool tail_starts(int total, int warps)
