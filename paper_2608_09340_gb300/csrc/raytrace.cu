@@ -538,6 +538,138 @@ __global__ void __launch_bounds__(kTraceBlock, MINB) k_trace_cube(const RayArgs 
     }
 }
 
+// One cell's extinction and emissivity for a lane's four channels, as two
+// pairs. FULL (n_ch = 4 LPR, rows 16-byte aligned): lane `sub` of a ray holds
+// channels 4 sub .. 4 sub + 3, read as one 16-byte vector per row, so a
+// ray's lanes read each row in one contiguous sweep. Otherwise pair h holds
+// channels sub + LPR (2h) and sub + LPR (2h + 1); channels past n_ch read zeros
+// (dtau = 0 and no intensity).
+template <int LPR, bool FULL>
+__device__ __forceinline__ void ray_rows(const RayArgs& A, int c, int sub, float2 (&v)[2], float2 (&j)[2])
+{
+    const float* arow = A.hcube + (size_t)c * A.n_ch;
+    const float* jrow = A.emiss + (size_t)c * A.n_ch;
+    if constexpr (FULL) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(arow) + sub);
+        const float4 e = __ldg(reinterpret_cast<const float4*>(jrow) + sub);
+        v[0] = make_float2(a.x, a.y);
+        v[1] = make_float2(a.z, a.w);
+        j[0] = make_float2(e.x, e.y);
+        j[1] = make_float2(e.z, e.w);
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int ka = sub + LPR * (2 * h), kb = ka + LPR;
+            v[h] = make_float2(ka < A.n_ch ? __ldg(arow + ka) : 0.0f, kb < A.n_ch ? __ldg(arow + kb) : 0.0f);
+            j[h] = make_float2(ka < A.n_ch ? __ldg(jrow + ka) : 0.0f, kb < A.n_ch ? __ldg(jrow + kb) : 0.0f);
+        }
+    }
+}
+
+// Channel of element e of pair h of lane `sub` (the layout of ray_rows).
+template <int LPR, bool FULL>
+__device__ __forceinline__ int lane_channel(int sub, int h, int e)
+{
+    return FULL ? 4 * sub + 2 * h + e : sub + LPR * (2 * h + e);
+}
+
+// The trace over the per-camera cube with LPR lanes per ray, 4 channels per
+// lane: a ray's lanes read a cell's row in one sweep, whatever cells the
+// neighbouring rays are in. For images whose pixels are far apart in cells,
+// or too few for a lane per ray and 4 or 8 channels (launch_trace_any): there
+// the lanes of k_trace_cube read separate rows, 4 to 16 bytes of each
+// 32-byte sector. Bound by the rows' sectors in L2.
+template <int LPR, bool JL, bool FULL>
+__global__ void __launch_bounds__(256, 4) k_trace_rows(const RayArgs A)
+{
+    constexpr int CPL = 4;
+    const int lane = threadIdx.x & 31;
+    const int sub = lane % LPR;
+    const long long ray = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 / LPR) + lane / LPR;
+    const long long npix = (long long)A.npix_x * A.npix_y;
+    if (ray >= npix) return;                 // no warp-wide operations follow
+    const int ix = (int)(ray % A.npix_x);
+    const int iy = (int)(ray / A.npix_x);
+
+    // the ray's start (k_ray_setup): first cell, position in it, hit
+    const float4 r0 = __ldg(A.rayinit + 2 * ray), r1 = __ldg(A.rayinit + 2 * ray + 1);
+    // the lane's channel pairs: intensity, optical depth in front of the
+    // segment, and their compensation terms
+    float2 I[CPL / 2], Ic[CPL / 2], tau[CPL / 2], tc[CPL / 2];
+#pragma unroll
+    for (int h = 0; h < CPL / 2; ++h) I[h] = Ic[h] = tau[h] = tc[h] = make_float2(0.0f, 0.0f);
+
+    if (__float_as_int(r0.w)) {
+        // cell and in-cell position as scalars (an array indexed by the
+        // crossing axis would live in local memory); the crossing axis is
+        // applied by selects
+        int ci0 = __float_as_int(r0.x), ci1 = __float_as_int(r0.y), ci2 = __float_as_int(r0.z);
+        float p0 = r1.x, p1 = r1.y, p2 = r1.z;
+        const float d0 = A.dirf[0], d1 = A.dirf[1], d2 = A.dirf[2];
+        const int nx = A.nx, ny = A.ny, nz = A.nz, nxy = A.nx * A.ny;
+        // the ray's start can lie outside (a ray along the box's face); after
+        // that only the axis just stepped on can leave the box
+        const bool inside = ci0 >= 0 && ci0 < nx && ci1 >= 0 && ci1 < ny && ci2 >= 0 && ci2 < nz;
+        const unsigned fwd = (d0 > 0.0f ? 1u : 0u) | (d1 > 0.0f ? 2u : 0u) | (d2 > 0.0f ? 4u : 0u);
+        const int max_seg = inside ? nx + ny + nz + 3 : 0;
+        int c = (ci2 * ny + ci1) * nx + ci0;
+        for (int seg = 0; seg < max_seg; ++seg) {
+            // distance to the face ahead on each axis, one FMA each
+            float s = fmaf(p0, A.face_neg[0], A.face_c[0]);
+            int axis = 0;
+            const float t1 = fmaf(p1, A.face_neg[1], A.face_c[1]);
+            if (t1 < s) { s = t1; axis = 1; }
+            const float t2 = fmaf(p2, A.face_neg[2], A.face_c[2]);
+            if (t2 < s) { s = t2; axis = 2; }
+            float2 v[2], j[2];
+            ray_rows<LPR, FULL>(A, c, sub, v, j);
+            float a0 = 0.0f, ta = 0.0f, jl = 0.0f;
+            if (JL) {
+                a0 = __ldg(A.cells + c).x;
+                ta = A.tau_abs ? __ldg(A.tau_abs + c) : 0.0f;
+                jl = __ldg(A.jline + c) * 0.56418958354775628f;
+            }
+            const float2 s2 = make_float2(s, s);
+#pragma unroll
+            for (int h = 0; h < CPL / 2; ++h) {
+                float2 vv = v[h], jj = j[h];
+                if (JL) {
+                    jj = __ffma2_rn(make_float2(jl, jl), vv, jj);
+                    vv = __ffma2_rn(make_float2(a0, a0), vv, make_float2(ta, ta));
+                }
+                const float2 dtau = __fmul2_rn(vv, s2);
+                const float2 T = exp_neg2(tau[h]);
+                kahan_add2(I[h], Ic[h], __fmul2_rn(__fmul2_rn(__fmul2_rn(T, jj), s2), escape_factor2(dtau)));
+                kahan_add2(tau[h], tc[h], dtau);
+            }
+            // move to the face, then step across it (the crossing axis is set exactly)
+            p0 = __saturatef(fmaf(s, d0, p0));
+            p1 = __saturatef(fmaf(s, d1, p1));
+            p2 = __saturatef(fmaf(s, d2, p2));
+            const bool x0 = axis == 0, x1 = axis == 1;
+            const bool up = (fwd >> axis) & 1u;
+            const int nc = (x0 ? ci0 : (x1 ? ci1 : ci2)) + (up ? 1 : -1);
+            const int dim = x0 ? nx : (x1 ? ny : nz);
+            if ((unsigned)nc >= (unsigned)dim) break;
+            const float pn = up ? 0.0f : 1.0f;
+            ci0 = x0 ? nc : ci0;
+            ci1 = x1 ? nc : ci1;
+            ci2 = (x0 || x1) ? ci2 : nc;
+            p0 = x0 ? pn : p0;
+            p1 = x1 ? pn : p1;
+            p2 = (x0 || x1) ? p2 : pn;
+            const int stride = x0 ? 1 : (x1 ? nx : nxy);
+            c += up ? stride : -stride;
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < CPL / 2; ++h) {
+        const int ka = lane_channel<LPR, FULL>(sub, h, 0), kb = lane_channel<LPR, FULL>(sub, h, 1);
+        if (ka < A.n_ch) A.maps[((size_t)ka * A.npix_y + iy) * A.npix_x + ix] = I[h].x;
+        if (kb < A.n_ch) A.maps[((size_t)kb * A.npix_y + iy) * A.npix_x + ix] = I[h].y;
+    }
+}
+
 // Without the per-camera cube (its memory not available): one warp per
 // pixel, the profile evaluated per segment.
 template <int CPL>
@@ -662,6 +794,32 @@ cudaError_t launch_trace(const RayArgs& A, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <int LPR>
+cudaError_t launch_rows(const RayArgs& A, cudaStream_t s)
+{
+    const long long npix = (long long)A.npix_x * A.npix_y;
+    const long long blocks = (npix * LPR + 255) / 256;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(A.emiss) | reinterpret_cast<uintptr_t>(A.hcube);
+    const bool full = A.n_ch == 4 * LPR && (at & 15u) == 0;
+    if (A.jline) {
+        if (full) k_trace_rows<LPR, true, true><<<(unsigned)blocks, 256, 0, s>>>(A);
+        else k_trace_rows<LPR, true, false><<<(unsigned)blocks, 256, 0, s>>>(A);
+    } else {
+        if (full) k_trace_rows<LPR, false, true><<<(unsigned)blocks, 256, 0, s>>>(A);
+        else k_trace_rows<LPR, false, false><<<(unsigned)blocks, 256, 0, s>>>(A);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rows_any(const RayArgs& A, cudaStream_t s)
+{
+    if (A.n_ch <= 16) return launch_rows<4>(A, s);
+    if (A.n_ch <= 32) return launch_rows<8>(A, s);
+    if (A.n_ch <= 64) return launch_rows<16>(A, s);
+    return launch_rows<32>(A, s);
+}
+
 // Channels per lane: the most of 8, 4, 2, 1 that pad the channels by at most
 // a quarter and leave enough lanes to hide the latency of the reads, about 50
 // warps per SM (fewer channels per lane repeat the geometry's work for more
@@ -669,22 +827,41 @@ cudaError_t launch_trace(const RayArgs& A, cudaStream_t s)
 // channels x 256^3 cells 19.5 with 8 (22.2 with 4, in ms); 400^2 x 16 x 128^3
 // 633 / 655 / 1040 with 8 / 4 / 2; 256^2 x 10 x 64^3 228 / 174 / 166 / 226
 // with 8 / 4 / 2 / 1; 128^2 x 5 x 128^3 264 / 252 / 203 / 179.
+// With more than 12 channels, a ray's lanes share its rows instead
+// (k_trace_rows) where lanes of their own would read small pieces of rows far
+// apart: one or two channels per lane, unless the image is so small that only
+// latency counts; unaligned rows with pixels more than 0.4 cells apart; four
+// channels per lane with pixels more than 0.8 cells apart, 0.5 if a row is
+// longer than a 128-byte line. Measured, us per call, calls back to back,
+// lanes of their own / shared rows: 150^2 x 32 x 100^3 715 / 262 (2 channels),
+// 100^2 x 64 x 48^3 208 / 100 (2), 220^2 x 16 x 128^3 529 / 287 (2), 100^2 x
+// 85 x 100^3 1057 / 456 (2), 450^2 x 85 x 200^3 9720 / 7485 (8, unaligned),
+// 220^2 x 32 x 200^3 1679 / 1304 (4). Eight aligned channels per lane read
+// whole sectors and win at any distance seen (220^2 x 64 x 200^3: 1648, 2451
+// with shared rows).
 cudaError_t launch_trace_any(const RayArgs& A, int sm_count, cudaStream_t s)
 {
     const long long npix = (long long)A.npix_x * A.npix_y, enough = (long long)sm_count * 1640;
     const uintptr_t at = reinterpret_cast<uintptr_t>(A.emiss) | reinterpret_cast<uintptr_t>(A.hcube);
+    const bool many = A.n_ch > 12;
     auto fits = [&](int cpl) {
         const int nb = (A.n_ch + cpl - 1) / cpl;
         return 4 * nb * cpl <= 5 * A.n_ch && npix * nb >= enough;
     };
     if (fits(8)) {
         if (A.n_ch % 8 == 0 && (at & 31u) == 0) return launch_trace<8, 2, 5, true>(A, s);
-        if (A.n_ch % 4 || (at & 15u)) return launch_trace<8, 2, 4, false>(A, s);
+        if (A.n_ch % 4 || (at & 15u)) {
+            if (many && A.pix > 0.4) return launch_rows_any(A, s);
+            return launch_trace<8, 2, 4, false>(A, s);
+        }
     }
     if (fits(4)) {
-        if (A.n_ch % 4 == 0 && (at & 15u) == 0) return launch_trace<4, 2, 6, true>(A, s);
+        const bool vec = A.n_ch % 4 == 0 && (at & 15u) == 0;
+        if (many && A.pix > (!vec ? 0.4 : A.n_ch > 32 ? 0.5 : 0.8)) return launch_rows_any(A, s);
+        if (vec) return launch_trace<4, 2, 6, true>(A, s);
         return launch_trace<4, 2, 6, false>(A, s);
     }
+    if (many && (A.n_ch > 16 || npix * A.n_ch > (long long)sm_count * 1100)) return launch_rows_any(A, s);
     if (fits(2)) return launch_trace<2, 4, 8, false>(A, s);
     return launch_trace<1, 4, 8, false>(A, s);
 }
