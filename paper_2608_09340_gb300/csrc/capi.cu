@@ -748,7 +748,9 @@ krl_status krl_run_packets(krl_grid* g, uint64_t n, uint64_t first_id, uint64_t 
     TransportArgs A{};
     fill_args(g, A, n, first_id, seed, T, records);
     A.ph_mode = mode;
-    A.even_fill = n <= (uint64_t)grid * (uint64_t)T.block;
+    // (walks with per-segment tallies are of few events: they keep full warps,
+    // and with them the rounds at which a visit's FP32 sums are flushed)
+    A.even_fill = !(f & F_SEG) && n <= (uint64_t)grid * (uint64_t)T.block;
     const int slot = (int)(g->run_seq.fetch_add(1u, std::memory_order_relaxed) % kSlots);
     unsigned long long* slot_stats = g->run_stats + (size_t)slot * ST_N;
     unsigned long long* slot_next = g->next + slot;
