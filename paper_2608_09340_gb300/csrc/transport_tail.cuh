@@ -415,20 +415,25 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
             return ((bits >> s0) | (s0 ? bits << (G - s0) : 0u)) & group;
         };
         stop = order(stop);
-        unsigned lost = 0u;
+        // A scattering without its row still has its own profile and place, so
+        // a crossing, absorption or destruction there stands, its outcome does
+        // not. The place after one beyond |x| = 300 was evaluated with another
+        // frequency than the packet has: nothing from there on stands.
+        unsigned lost = 0u, wrong = 0u;
         if (__any_sync(kFull, pos < now && (out || far))) {     // rare
             lost = order(__ballot_sync(kFull, pos < now && out) >> base);
-            lost |= order(__ballot_sync(kFull, pos < now && far) >> base) << 1;
+            wrong = order(__ballot_sync(kFull, pos < now && far) >> base) << 1;
         }
         int lim = room < (uint32_t)now ? (int)room : now;
-        const int fo = lost ? __ffs(lost) - 1 : 64;     // its profile and place are right, its outcome is not
+        const int fo = lost ? __ffs(lost) - 1 : 64, fw = wrong ? __ffs(wrong) - 1 : 64;
         int f = stop ? __ffs(stop) - 1 : now;
+        if (fw < lim) lim = fw;
         const bool ends = f < lim && f <= fo;           // segment f runs, and is not a plain scattering
         if (fo < lim) lim = fo;
         f = alive ? (f < lim ? f : lim) : 0;            // (a group without a packet keeps known >= 0)
         have -= f;
         known -= f;
-        if (!ends && f == fo) {                         // draw again, the window around x
+        if (!ends && (f == fo || f == fw)) {            // draw again, the window around x
             have = known = 0;
             ev = 0;
         }
