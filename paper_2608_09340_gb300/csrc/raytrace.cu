@@ -26,7 +26,10 @@
 // that FP32 stays within 1e-5 of an FP64 trace over hundreds of segments.
 #include <math.h>
 
+#include <type_traits>
+
 #include "krl_internal.cuh"
+#include "trace_tile.cuh"
 
 namespace krl {
 
@@ -376,12 +379,11 @@ __device__ __forceinline__ void cell_rows(const RayArgs& A, int c, int k0, float
     }
 }
 
-constexpr int kTileX = 8, kTileY = 4;       // a warp's pixels
 constexpr int kTraceBlock = 128;
 
 // The trace over the per-camera cube (k_rt_profile). A warp follows the rays
-// of 8 x 4 neighbouring pixels, one per lane, for the same CPL channels; the
-// channel blocks of a tile are neighbouring CTAs. The lanes' cells nearly
+// of 8 x 4 neighbouring pixels (trace_tile.cuh), one per lane, for the same
+// CPL channels; the channel blocks of a tile are neighbouring CTAs. The lanes' cells nearly
 // coincide (pixels oversample the cells), so their reads share sectors and
 // their optical depths are alike: a line a few thermal widths wide touches a
 // block of channels in a small part of the cells, and elsewhere the warp
@@ -395,17 +397,22 @@ constexpr int kTraceBlock = 128;
 // special-function slots; in this layout 16.
 // The cube holds the extinction alpha0 H + alpha_abs (JL false) or H (JL true:
 // the line-emission term needs H; alpha is formed here).
-template <int CPL, int D, int MINB, bool JL, bool VEC>
-__global__ void __launch_bounds__(kTraceBlock, MINB) k_trace_cube(const RayArgs A, int tiles_x, int blocks_ch)
+// STRIP: a tile of other than 8 x 4 pixels (instantiations of their own: with
+// the shape at run time in one kernel the 8 x 4 case took 1.2 % longer).
+template <int CPL, int D, int MINB, bool JL, bool VEC, bool STRIP>
+__global__ void __launch_bounds__(kTraceBlock, MINB) k_trace_cube(const RayArgs A, int tiles_x, int blocks_ch, int strip_bits)
 {
+    const int tile_bits = STRIP ? strip_bits : 3;
     constexpr int HP = (CPL + 1) / 2;
     const int lane = threadIdx.x & 31;
     const int k0 = (int)(blockIdx.x % (unsigned)blocks_ch) * CPL;
     const long long tile = (long long)(blockIdx.x / (unsigned)blocks_ch) * (kTraceBlock / 32) + (threadIdx.x >> 5);
-    // lanes in Z order: a wide load serves 4 or 8 lanes at a time, which then
-    // are 2 x 2 or 4 x 2 pixels and mostly one cell
-    const int ix = (int)(tile % tiles_x) * kTileX + ((lane & 1) | (lane >> 1 & 2) | (lane >> 2 & 4));
-    const long long iyl = tile / tiles_x * kTileY + ((lane >> 1 & 1) | (lane >> 2 & 2));
+    // a wide load serves 4 or 8 lanes at a time, which lie next to one another
+    // in the tile and mostly in one cell
+    int lx, ly;
+    trace_tile_place(lane, tile_bits, &lx, &ly);
+    const int ix = (int)(((tile % tiles_x) << tile_bits) + lx);
+    const long long iyl = tile / tiles_x * (32 >> tile_bits) + ly;
     const bool pixel = ix < A.npix_x && iyl < A.npix_y;
     const int iy = (int)iyl;
 
@@ -784,13 +791,22 @@ __global__ void __launch_bounds__(256) k_raytrace(const RayArgs A)
 template <int CPL, int D, int MINB, bool VEC>
 cudaError_t launch_trace(const RayArgs& A, cudaStream_t s)
 {
-    const int tiles_x = (A.npix_x + kTileX - 1) / kTileX;
-    const long long tiles = (long long)tiles_x * ((A.npix_y + kTileY - 1) / kTileY);
+    const int tile_bits = trace_tile_bits(A.npix_x, A.npix_y);
+    const int tiles_x = (int)trace_tiles_x(A.npix_x, tile_bits);
+    const long long tiles = tiles_x * trace_tiles_y(A.npix_y, tile_bits);
     const int blocks_ch = (A.n_ch + CPL - 1) / CPL;
     const long long blocks = (tiles + kTraceBlock / 32 - 1) / (kTraceBlock / 32) * blocks_ch;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    if (A.jline) k_trace_cube<CPL, D, MINB - (CPL == 8 && VEC ? 1 : 0), true, VEC><<<(unsigned)blocks, kTraceBlock, 0, s>>>(A, tiles_x, blocks_ch);
-    else k_trace_cube<CPL, D, MINB, false, VEC><<<(unsigned)blocks, kTraceBlock, 0, s>>>(A, tiles_x, blocks_ch);
+    auto launch = [&](auto strip) {
+        constexpr bool S = decltype(strip)::value;
+        if (A.jline)
+            k_trace_cube<CPL, D, MINB - (CPL == 8 && VEC ? 1 : 0), true, VEC, S>
+                <<<(unsigned)blocks, kTraceBlock, 0, s>>>(A, tiles_x, blocks_ch, tile_bits);
+        else
+            k_trace_cube<CPL, D, MINB, false, VEC, S><<<(unsigned)blocks, kTraceBlock, 0, s>>>(A, tiles_x, blocks_ch, tile_bits);
+    };
+    if (tile_bits == 3) launch(std::false_type());
+    else launch(std::true_type());
     return cudaGetLastError();
 }
 
