@@ -75,7 +75,7 @@ __device__ __forceinline__ float voigt_rt(float x, const ProfileTables<PAIRS>& P
 {
     float ax = fabsf(x);
     if (ax < 1e-4f) return H0;
-    if (ax > 1e3f) return a / (1.7724538509055160f * ax * ax) * (1.0f + 1.5f / (ax * ax));
+    if (!(ax <= 1e3f)) return a / (1.7724538509055160f * ax * ax) * (1.0f + 1.5f / (ax * ax));    // (or NaN)
     // ax = m 2^e, m in [0.5, 1): ax is a normal number here, so from its bits
     const unsigned bits = __float_as_uint(ax);
     const float m = __uint_as_float((bits & 0x007fffffu) | 0x3f000000u);
@@ -329,6 +329,14 @@ __device__ __forceinline__ float2 exp_neg2(float2 x)
     return r;
 }
 
+// The larger one, or NaN if either is.
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
 // (1 - e^{-d})/d of two values without a branch: from e^{-d} above d = 0.05,
 // else its Taylor series 1 - d/2 + d^2/6 - d^3/24 + d^4/120 (Horner in d)
 __device__ __forceinline__ float2 escape_series2(float2 d)
@@ -519,13 +527,13 @@ __global__ void __launch_bounds__(kTraceBlock, MINB) k_trace_cube(const RayArgs 
 #pragma unroll
         for (int h = 0; h < HP; ++h) {
             dt[h] = __fmul2_rn(v[h], s2);
-            dmax = fmaxf(dmax, fmaxf(dt[h].x, dt[h].y));
+            dmax = max_nan(dmax, max_nan(dt[h].x, dt[h].y));
         }
         float2 tj[HP];          // T j s
 #pragma unroll
         for (int h = 0; h < HP; ++h) tj[h] = __fmul2_rn(__fmul2_rn(T[h], j[h]), s2);
-        if (__any_sync(0xffffffffu, dmax > 5e-8f)) {            // warp-uniform
-            if (__any_sync(0xffffffffu, dmax > 0.05f)) {
+        if (__any_sync(0xffffffffu, !(dmax <= 5e-8f))) {        // warp-uniform; NaN takes the full formula
+            if (__any_sync(0xffffffffu, !(dmax <= 0.05f))) {
 #pragma unroll
                 for (int h = 0; h < HP; ++h) tj[h] = __fmul2_rn(tj[h], escape_factor2(dt[h]));
             } else {
