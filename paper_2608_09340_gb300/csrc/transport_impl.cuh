@@ -1013,7 +1013,7 @@ __global__ void __launch_bounds__(kDepositBlock, 5) k_emiss_deposit(const __grid
                 const int k = __float_as_int(sa.x) + (e - __float_as_int(sb.w));
                 const float kf = __int_as_float(0x4B000000 + k) - 8388608.0f;      // (float)k, k < 2^23
                 const float D = emiss_delta<float>(T, sa.z, kf);
-                const bool near = on && fabsf(D) <= (float)kRdMax;
+                const bool near = on && !(fabsf(D) > (float)kRdMax);       // (NaN counts, as in emiss_channel)
                 float val = 0.0f;
                 const bool table = near && T.cell >= 0;
                 int node = 0;
