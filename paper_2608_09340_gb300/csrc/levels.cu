@@ -201,7 +201,9 @@ __global__ void __launch_bounds__(128) k_solve(LevelConst L, const double* gamma
             change = fmax(change, fabs(v - old));
             *p = v;
         }
-        change = nm > 0.0 ? change / nm : 0.0;            // rounding is monotonic: the largest of the quotients
+        // (rounding is monotonic: the largest of the quotients; an infinite
+        // density has none)
+        change = nm > 0.0 && nm < (double)INFINITY ? change / nm : 0.0;
         // (most cells change less than some other has: no atomic for them)
         const unsigned long long bits = (unsigned long long)__double_as_longlong(change);
         if (max_change && bits > *(volatile unsigned long long*)max_change) atomicMax(max_change, bits);
