@@ -1120,7 +1120,7 @@ krl_status krl_levels_solve(krl_grid* g, const krl_levels_desc* d, const double*
     ls = level_scratch(g, s);
     if (ls != KRL_OK) return ls;
     KRL_CUDA(cudaMemsetAsync(g->lv_change, 0, sizeof(unsigned long long), s), "levels");
-    KRL_CUDA(levels_solve(L, gamma, g->ncell, g->n_coll, d->n_mol, pops, g->lv_change, s), "levels solve");
+    KRL_CUDA(levels_solve(L, gamma, g->ncell, g->n_coll, d->n_mol, pops, g->lv_change, g->num_sms, s), "levels solve");
     if (max_change) {
         unsigned long long bits = 0;
         KRL_CUDA(cudaMemcpyAsync(&bits, g->lv_change, 8, cudaMemcpyDeviceToHost, s), "levels");
@@ -1144,7 +1144,7 @@ krl_status krl_levels_iterate(krl_grid* g, const krl_levels_desc* d, int n_iter,
     if (ls != KRL_OK) return ls;
     const int ncell = g->ncell;
     const size_t n = (size_t)ncell;
-    if (init_lte) KRL_CUDA(levels_lte(L, d->n_mol, ncell, pops, s), "levels lte");
+    if (init_lte) KRL_CUDA(levels_lte(L, d->n_mol, ncell, pops, g->num_sms, s), "levels lte");
     KRL_CUDA(cudaMemcpyAsync(g->lv_pops0, pops, n * L.n * sizeof(double), cudaMemcpyDeviceToDevice, s), "levels");
     for (int it = 0; it < n_iter; ++it) {
         for (int t = 0; t < L.n_trans; ++t) {
@@ -1178,7 +1178,7 @@ krl_status krl_levels_iterate(krl_grid* g, const krl_levels_desc* d, int n_iter,
                      "gamma");
         }
         KRL_CUDA(cudaMemsetAsync(g->lv_change, 0, sizeof(unsigned long long), s), "levels");
-        KRL_CUDA(levels_solve(L, g->lv_gamma, ncell, g->n_coll, d->n_mol, pops, g->lv_change, s), "levels solve");
+        KRL_CUDA(levels_solve(L, g->lv_gamma, ncell, g->n_coll, d->n_mol, pops, g->lv_change, g->num_sms, s), "levels solve");
         if (max_change) {
             unsigned long long bits = 0;
             KRL_CUDA(cudaMemcpyAsync(&bits, g->lv_change, 8, cudaMemcpyDeviceToHost, s), "levels");

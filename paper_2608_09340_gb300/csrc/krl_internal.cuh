@@ -247,7 +247,7 @@ struct LevelConst {
     int n_trans;                        // radiative pairs, ordered by (l, u)
     int tu[kMaxTrans], tl[kMaxTrans];
 };
-cudaError_t levels_lte(const LevelConst& L, const float* n_mol, int ncell, double* pops, cudaStream_t s);
+cudaError_t levels_lte(const LevelConst& L, const float* n_mol, int ncell, double* pops, int sm_count, cudaStream_t s);
 cudaError_t levels_field(const double* pops, int ncell, int n_lev, int lev, double scale, float* out, cudaStream_t s);
 // total: device scratch of levels_sum_scratch_doubles() doubles; the sum lands in total[0].
 size_t levels_sum_scratch_doubles();
@@ -255,7 +255,7 @@ cudaError_t levels_sum_rate(const double* pops, int ncell, int n_lev, int u, dou
 cudaError_t levels_gamma(const double* exc, int ncell, const double* total, double dx, double sigma0, double n_packets,
                          double* gamma, cudaStream_t s);
 cudaError_t levels_solve(const LevelConst& L, const double* gamma, int ncell, const float* n_coll, const float* n_mol,
-                         double* pops, unsigned long long* max_change, cudaStream_t s);
+                         double* pops, unsigned long long* max_change, int sm_count, cudaStream_t s);
 
 // ---------------------------------------------------------------- setup kernels (tables.cu)
 struct LineTables {

@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(256) k_lte(LevelConst L, const float* n_mol, i
     __syncthreads();
     double z = 0.0;
     for (int i = 0; i < L.n; ++i) z += w[i];
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
+    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)ncell; c += gridDim.x * blockDim.x) {
         const double nm = (double)n_mol[c];
         for (int i = 0; i < L.n; ++i) pops[(size_t)c * L.n + i] = nm * w[i] / z;
     }
@@ -123,11 +123,14 @@ __device__ __forceinline__ void eliminate(double (&M)[N][N + 1])
 
 // One thread per cell, N levels. What the cells share, the detailed-balance
 // factors and the ratios of degeneracies of each pair, is formed once per
-// block; the matrices are unrolled over N, so that they live in registers and
-// the pivoting is selects. Bound by the FP64 pipe (2 lanes per clock and SM):
-// 16 divisions and about 200 other operations per cell at 5 levels. 128^3
-// cells: 2.8 -> 1.34 ms; before, each cell formed the exponentials and ratios
-// (20 of each) itself, and the matrices lived in local memory.
+// block; the matrices are unrolled over N, so that they live in registers (with
+// 3 levels 8 bytes of spills, with 8 levels 112) and the pivoting
+// is selects. Bound by the FP64 pipe (2 lanes per clock and SM): 16 divisions
+// and about 200 other operations per cell at 5 levels. 128^3 cells, 5 levels:
+// 2.8 -> 1.34 ms; before, each cell formed the exponentials and ratios (20 of
+// each) itself, and the matrices lived in local memory. Whole calls with 2, 3,
+// 4, 5, 6, 7 and 8 levels: 1.39, 1.47, 2.06, 3.10, 4.39, 5.94 and 7.74 ms
+// before, 0.30, 0.53, 0.87, 1.43, 1.86, 2.51 and 3.30 now.
 template <int N>
 __global__ void __launch_bounds__(128) k_solve(LevelConst L, const double* gamma, int ncell, const float* n_coll,
                                                const float* n_mol, double* pops, unsigned long long* max_change)
@@ -147,7 +150,7 @@ __global__ void __launch_bounds__(128) k_solve(LevelConst L, const double* gamma
         }
     }
     __syncthreads();
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
+    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)ncell; c += gridDim.x * blockDim.x) {
         double R[N][N];
         const double nc = n_coll ? (double)n_coll[c] : 0.0;
 #pragma unroll
@@ -210,25 +213,25 @@ __global__ void __launch_bounds__(128) k_solve(LevelConst L, const double* gamma
     }
 }
 
-// Blocks of a grid-stride kernel that shares set-up per block.
-int stride_blocks(int ncell, int threads)
+// Blocks of a grid-stride kernel that shares set-up per block: 16 per SM.
+int stride_blocks(int ncell, int threads, int sm_count)
 {
-    const int full = (ncell + threads - 1) / threads;
-    return full < 152 * 16 ? full : 152 * 16;
+    const int full = (int)(((unsigned)ncell + threads - 1) / threads);
+    return full < sm_count * 16 ? full : sm_count * 16;
 }
 
 template <int N>
 void launch_solve(const LevelConst& L, const double* gamma, int ncell, const float* n_coll, const float* n_mol, double* pops,
-                  unsigned long long* max_change, cudaStream_t s)
+                  unsigned long long* max_change, int sm_count, cudaStream_t s)
 {
-    k_solve<N><<<stride_blocks(ncell, 128), 128, 0, s>>>(L, gamma, ncell, n_coll, n_mol, pops, max_change);
+    k_solve<N><<<stride_blocks(ncell, 128, sm_count), 128, 0, s>>>(L, gamma, ncell, n_coll, n_mol, pops, max_change);
 }
 
 }  // namespace
 
-cudaError_t levels_lte(const LevelConst& L, const float* n_mol, int ncell, double* pops, cudaStream_t s)
+cudaError_t levels_lte(const LevelConst& L, const float* n_mol, int ncell, double* pops, int sm_count, cudaStream_t s)
 {
-    k_lte<<<stride_blocks(ncell, 256), 256, 0, s>>>(L, n_mol, ncell, pops);
+    k_lte<<<stride_blocks(ncell, 256, sm_count), 256, 0, s>>>(L, n_mol, ncell, pops);
     return cudaGetLastError();
 }
 
@@ -255,16 +258,16 @@ cudaError_t levels_gamma(const double* exc, int ncell, const double* total, doub
 }
 
 cudaError_t levels_solve(const LevelConst& L, const double* gamma, int ncell, const float* n_coll, const float* n_mol,
-                         double* pops, unsigned long long* max_change, cudaStream_t s)
+                         double* pops, unsigned long long* max_change, int sm_count, cudaStream_t s)
 {
     switch (L.n) {
-    case 2: launch_solve<2>(L, gamma, ncell, n_coll, n_mol, pops, max_change, s); break;
-    case 3: launch_solve<3>(L, gamma, ncell, n_coll, n_mol, pops, max_change, s); break;
-    case 4: launch_solve<4>(L, gamma, ncell, n_coll, n_mol, pops, max_change, s); break;
-    case 5: launch_solve<5>(L, gamma, ncell, n_coll, n_mol, pops, max_change, s); break;
-    case 6: launch_solve<6>(L, gamma, ncell, n_coll, n_mol, pops, max_change, s); break;
-    case 7: launch_solve<7>(L, gamma, ncell, n_coll, n_mol, pops, max_change, s); break;
-    case 8: launch_solve<8>(L, gamma, ncell, n_coll, n_mol, pops, max_change, s); break;
+    case 2: launch_solve<2>(L, gamma, ncell, n_coll, n_mol, pops, max_change, sm_count, s); break;
+    case 3: launch_solve<3>(L, gamma, ncell, n_coll, n_mol, pops, max_change, sm_count, s); break;
+    case 4: launch_solve<4>(L, gamma, ncell, n_coll, n_mol, pops, max_change, sm_count, s); break;
+    case 5: launch_solve<5>(L, gamma, ncell, n_coll, n_mol, pops, max_change, sm_count, s); break;
+    case 6: launch_solve<6>(L, gamma, ncell, n_coll, n_mol, pops, max_change, sm_count, s); break;
+    case 7: launch_solve<7>(L, gamma, ncell, n_coll, n_mol, pops, max_change, sm_count, s); break;
+    case 8: launch_solve<8>(L, gamma, ncell, n_coll, n_mol, pops, max_change, sm_count, s); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
