@@ -366,6 +366,7 @@ void fill_args(const krl_grid* g, TransportArgs& A, uint64_t n, uint64_t first_i
     A.max_iters = T.max_iters;
     A.max_iters32 = (unsigned)T.max_iters;        // resolve_tune keeps it below 2^32
     A.refill_min = T.refill_min;
+    A.tail_warps = transport_tail_warps((L.tally_flags & KRL_TALLY_EMISS) != 0);
     A.tau_abs = g->tau_abs;
     A.absw = g->absw;
     A.ph_mode = g->line.ph_mode;
@@ -1025,11 +1026,15 @@ krl_status krl_batch_run(krl_batch* b, const uint64_t* packets, const uint64_t* 
     std::vector<int> order(n);
     for (size_t m = 0; m < n; ++m) order[m] = (int)m;
     std::stable_sort(order.begin(), order.end(), [packets](int x, int y) { return packets[x] > packets[y]; });
+    bool emiss = false;
+    for (const krl_grid* g : b->grids) emiss = emiss || (g->line.tally_flags & KRL_TALLY_EMISS);
+    const int tail_warps = transport_tail_warps(emiss);
     for (size_t k = 0; k < n; ++k) {
         const int m = order[k];
         TransportArgs& A = b->h_args[k];
         A = TransportArgs{};
         fill_args(b->grids[m], A, packets[m], first_ids ? first_ids[m] : 0, seed, T, records ? records[m] : nullptr);
+        A.tail_warps = tail_warps;
         A.next = b->d_counts + m;
         A.stats = b->d_counts + n + (size_t)m * ST_N;
     }
@@ -1037,7 +1042,7 @@ krl_status krl_batch_run(krl_batch* b, const uint64_t* packets, const uint64_t* 
              "upload model arguments");
     KRL_CUDA(cudaMemsetAsync(b->d_counts, 0, n * (1 + ST_N) * sizeof(unsigned long long), s), "reset counters");
     KRL_CUDA(cudaMemsetAsync(b->d_cursor, 0, sizeof(int), s), "reset cursor");
-    BatchArgs B{b->d_args, b->n, b->d_cursor, round_keys(seed)};
+    BatchArgs B{b->d_args, b->n, b->d_cursor, round_keys(seed), tail_warps};
     KRL_CUDA(launch_transport_batch(B, T.precision, f, grid, T.block, s), "batch launch");
     KRL_CUDA(add_counters_batch(b->d_dst, b->d_counts + n, b->n, s), "accumulate counters");
     if (stats) {

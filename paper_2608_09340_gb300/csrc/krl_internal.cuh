@@ -142,6 +142,7 @@ struct TransportArgs {
     unsigned long long max_iters;
     unsigned max_iters32;     // min(max_iters, 2^32 - 1): the per-event check in 32 bits
     int refill_min;           // 0: the walk chooses
+    int tail_warps;           // warps of a CTA that walk its last packets by groups of lanes
     int even_fill;            // no more packets than lanes in the grid: equal shares, no work counter
     // line-profile mode (krl_line_desc.ph_mode: 2, or 1 / 3 below)
     int ph_mode;
@@ -188,6 +189,7 @@ struct BatchArgs {
     int n_models;
     int* cursor;                   // device: lowest model that may still have work
     RoundKeys keys;                // one seed for every model of the batch
+    int tail_warps;                // of every model
 };
 cudaError_t launch_transport_batch(const BatchArgs& B, int precision, unsigned features, int grid, int block,
                                    cudaStream_t s);
@@ -202,6 +204,8 @@ int transport_occupancy_ph(int ph_mode, int precision, unsigned features, int bl
 int transport_max_block(int precision, unsigned features);
 // CTA of the F_WIDE walk (FP32, profile mode 2).
 int transport_wide_block(unsigned features);
+// TransportArgs::tail_warps of a run with (or without) an emissivity tally.
+int transport_tail_warps(bool emiss);
 // The batched launch: its CTA size limit and occupancy.
 int transport_batch_max_block();
 int transport_batch_occupancy(int precision, unsigned features, int block);

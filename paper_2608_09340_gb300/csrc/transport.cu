@@ -47,6 +47,8 @@ int transport_max_block(int precision, unsigned features)
 
 int transport_wide_block(unsigned features) { return features & F_RICH ? kLightBlock : kLeanBlock; }
 
+int transport_tail_warps(bool emiss) { return emiss ? kTailWarpsL1 : kTailWarps; }
+
 int transport_occupancy(int precision, unsigned features, int block, int ph_mode)
 {
     if (ph_mode == 1 || ph_mode == 3 || ph_mode == 4) return transport_occupancy_ph(ph_mode, precision, features, block);

@@ -1098,7 +1098,7 @@ constexpr int stash_words() { return 8 + (sizeof(R) == 8 ? 1 : 0) + ((F & F_RICH
 
 // (the stash, or the buffers of the last packets' walk in its place)
 template <typename R, unsigned F>
-constexpr size_t smem_bytes(int block);
+constexpr size_t smem_bytes(int block, int tail_warps);
 
 template <typename R>
 __device__ __forceinline__ void put_r(uint32_t* w, int& f, int n, int slot, R v)
@@ -1455,11 +1455,15 @@ __device__ __forceinline__ bool advance(const TransportArgs& A, const RoundKeys&
 #include "transport_tail.cuh"
 
 template <typename R, unsigned F>
-constexpr size_t smem_bytes(int block)
+constexpr size_t smem_bytes(int block, int tail_warps)
 {
-    const size_t stash = (size_t)stash_words<R, F>() * 4u * (size_t)block;
-    return kStashOff + (sizeof(R) == 4 && tail_bytes(block) > stash ? tail_bytes(block) : stash);
+    const size_t stash = (size_t)stash_words<R, F>() * 4u * (size_t)block, tail = tail_bytes(block, tail_warps);
+    return kStashOff + (sizeof(R) == 4 && tail > stash ? tail : stash);
 }
+// (the splits of an SM's 256 KB: ... 164, 196 or 228 KB of shared memory, of
+// which each CTA takes 1 KB more than it asks for)
+static_assert(2 * (smem_bytes<float, F_RICH | F_SEG>(256, kTailWarpsL1) + 1024) <= 196 * 1024,
+              "two CTAs with an emissivity tally leave L1 60 KB");
 
 // One model's walk by the whole CTA: stage the model's tables in shared
 // memory, run packets until the model's id counter is exhausted and every
@@ -1634,7 +1638,7 @@ __device__ __forceinline__ void run_model(const TransportArgs& A, const RoundKey
             }
             if (total == 0) break;            // CTA-uniform
             if constexpr (sizeof(R) == 4 && (PH == 2 || PH == 4)) {
-                const int tw = nwarps < kTailWarps ? nwarps : kTailWarps;
+                const int tw = nwarps < A.tail_warps ? nwarps : A.tail_warps;
                 if (tail_starts(total, tw) && 2 * scatters > total) {     // CTA-uniform
                     // the last packets, dealt over tw warps: group g of warp
                     // w walks packet g tw + w
@@ -1756,9 +1760,9 @@ cudaError_t launch_one(const TransportArgs& A, int grid, int block, cudaStream_t
     // device: set it on every launch (a host-side call of about a
     // microsecond), so that a launch on any device of the process has it
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_bytes<R, F>(max_block<R, F>()));
+                                         (int)smem_bytes<R, F>(max_block<R, F>(), kTailWarps));
     if (e != cudaSuccess) return e;
-    kern<<<grid, block, smem_bytes<R, F>(block), s>>>(A);
+    kern<<<grid, block, smem_bytes<R, F>(block, A.tail_warps), s>>>(A);
     return cudaGetLastError();
 }
 
@@ -1768,9 +1772,9 @@ cudaError_t launch_batch_one(const BatchArgs& B, int grid, int block, cudaStream
     if (block > kBatchBlock) return cudaErrorInvalidConfiguration;
     auto kern = k_transport_batch<R, F>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_bytes<R, F>(kBatchBlock));   // per device: every launch
+                                         (int)smem_bytes<R, F>(kBatchBlock, kTailWarps));   // per device: every launch
     if (e != cudaSuccess) return e;
-    kern<<<grid, block, smem_bytes<R, F>(block), s>>>(B);
+    kern<<<grid, block, smem_bytes<R, F>(block, B.tail_warps), s>>>(B);
     return cudaGetLastError();
 }
 
@@ -1779,9 +1783,9 @@ int occupancy_one(int block)
 {
     if (block > max_block<R, F>()) return 0;
     auto kern = k_transport<R, F, PH>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<R, F>(max_block<R, F>()));
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<R, F>(max_block<R, F>(), kTailWarps));
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, block, smem_bytes<R, F>(block)) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, block, smem_bytes<R, F>(block, kTailWarps)) != cudaSuccess) return 0;
     return n;
 }
 
@@ -1790,9 +1794,9 @@ int batch_occupancy_one(int block)
 {
     if (block > kBatchBlock) return 0;
     auto kern = k_transport_batch<R, F>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<R, F>(kBatchBlock));
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<R, F>(kBatchBlock, kTailWarps));
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, block, smem_bytes<R, F>(block)) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, block, smem_bytes<R, F>(block, kTailWarps)) != cudaSuccess) return 0;
     return n;
 }
 

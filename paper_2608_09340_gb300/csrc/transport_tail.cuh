@@ -33,7 +33,17 @@
 // 1e5 packets 368 / 369 ms, static sphere 492 / 500, dusty slab 107 / 109,
 // 64 models 162 / 167, 1e4-packet slab 35.8 / 35.1; with groups of 4 from
 // 2 kTailWide down the slab (33 packets per CTA) took 52 for 44.
-constexpr int kTailWarps = 8;
+//
+// Runs with an emissivity tally (TransportArgs::tail_warps) use kTailWarpsL1:
+// a segment that the walk deposits itself reads the R_IIA table through L1,
+// and with 8 warps' buffers two CTAs need the SM's largest shared-memory
+// split, which leaves L1 28 of 256 KB; with 6 they leave it 60. Medians of 8
+// runs, without groups (17 KB for the stash) / 8 warps / 6: 128^3 envelope, 3
+// cameras x 64 channels, 1e6 packets deposited in the walk 20.3 / 27.0 / 22.0
+// ms, 4e6 with the default buffer 46.9 / 52.3 / 46.1, a box of tau0 = 100 with
+// 1e5 packets 32.3 / 40.7 / 33.4. Without that tally 8 are better (box of
+// tau0 = 1000 with mean intensity, 1e5 packets: 27.0 / 12.5 / 13.4).
+constexpr int kTailWarps = 8, kTailWarpsL1 = 6;
 constexpr int kTailWide = 4;
 constexpr bool tail_starts(int total, int warps)
 {
@@ -70,9 +80,9 @@ struct TailBuf {
 static_assert(sizeof(TailBuf) % 16 == 0, "warps' buffers stay aligned");
 static_assert(kUsNx * sizeof(float) <= sizeof(float4) * 32, "rows below a slot's window fall into a and b");
 
-constexpr size_t tail_bytes(int block)
+constexpr size_t tail_bytes(int block, int warps)
 {
-    const int w = block / 32 < kTailWarps ? block / 32 : kTailWarps;
+    const int w = block / 32 < warps ? block / 32 : warps;
     return (size_t)w * sizeof(TailBuf);
 }
 
