@@ -888,6 +888,10 @@ __device__ __forceinline__ bool append_segment(const TransportArgs& A, unsigned 
             // then fails and the new word is looked at (at most 31 times)
             unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(word);
             for (;;) {
+                if (old >= A.seg_cap) {         // the buffer is full: nothing to take
+                    first = old;
+                    break;
+                }
                 const unsigned left = (unsigned)(0ull - old) & (chunk - 1u);
                 const bool fits = cnt <= left;
                 first = fits ? old : atomicAdd(A.seg_count, (unsigned long long)chunk);
