@@ -749,6 +749,7 @@ krl_status krl_run_packets(krl_grid* g, uint64_t n, uint64_t first_id, uint64_t 
     TransportArgs A{};
     fill_args(g, A, n, first_id, seed, T, records);
     A.ph_mode = mode;
+    if (mode == 4) A.tail_warps = transport_tail_warps_constant(g->emiss != nullptr, n, grid);
     // (walks with per-segment tallies are of few events: they keep full warps,
     // and with them the rounds at which a visit's FP32 sums are flushed)
     A.even_fill = !(f & F_SEG) && n <= (uint64_t)grid * (uint64_t)T.block;

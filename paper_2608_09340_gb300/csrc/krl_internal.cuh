@@ -204,8 +204,10 @@ int transport_occupancy_ph(int ph_mode, int precision, unsigned features, int bl
 int transport_max_block(int precision, unsigned features);
 // CTA of the F_WIDE walk (FP32, profile mode 2).
 int transport_wide_block(unsigned features);
-// TransportArgs::tail_warps of a run with (or without) an emissivity tally.
+// TransportArgs::tail_warps of a run with (or without) an emissivity tally and
+// of one with its tables in the constant bank and n packets on so many CTAs.
 int transport_tail_warps(bool emiss);
+int transport_tail_warps_constant(bool emiss, unsigned long long n, int ctas);
 // The batched launch: its CTA size limit and occupancy.
 int transport_batch_max_block();
 int transport_batch_occupancy(int precision, unsigned features, int block);

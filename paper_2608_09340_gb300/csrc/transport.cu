@@ -49,6 +49,12 @@ int transport_wide_block(unsigned features) { return features & F_RICH ? kLightB
 
 int transport_tail_warps(bool emiss) { return emiss ? kTailWarpsL1 : kTailWarps; }
 
+int transport_tail_warps_constant(bool emiss, unsigned long long n, int ctas)
+{
+    const int w = transport_tail_warps(emiss);
+    return n <= (unsigned long long)ctas * (unsigned)(w * kTailWide) || w < kTailWarpsConst ? w : kTailWarpsConst;
+}
+
 int transport_occupancy(int precision, unsigned features, int block, int ph_mode)
 {
     if (ph_mode == 1 || ph_mode == 3 || ph_mode == 4) return transport_occupancy_ph(ph_mode, precision, features, block);

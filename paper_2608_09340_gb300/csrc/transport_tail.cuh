@@ -43,7 +43,14 @@
 // ms, 4e6 with the default buffer 46.9 / 52.3 / 46.1, a box of tau0 = 100 with
 // 1e5 packets 32.3 / 40.7 / 33.4. Without that tally 8 are better (box of
 // tau0 = 1000 with mean intensity, 1e5 packets: 27.0 / 12.5 / 13.4).
-constexpr int kTailWarps = 8, kTailWarpsL1 = 6;
+//
+// With the tables in the constant bank (mode 4) the lanes of a group read
+// different addresses, which that bank serves one after the other, so that
+// many groups stand in one another's way: kTailWarpsConst, unless a CTA's
+// packets all go to groups at once. Slab of 128 cells, tau = 32000, without
+// groups / 8 warps / 4: 2e3 packets 610 / 151 / 183 ms, 2e4 788 / 707 / 567,
+// 2e5 2496 / 2608 / 2421; dusty slab, 1e5 packets 104 / 113 / 100.
+constexpr int kTailWarps = 8, kTailWarpsL1 = 6, kTailWarpsConst = 4;
 constexpr int kTailWide = 4;
 constexpr bool tail_starts(int total, int warps)
 {
