@@ -200,9 +200,14 @@ typedef struct {
                                    (same walk in double, for lockstep checks)       */
     int block;                  /* threads per CTA, multiple of 32; at most 512 for
                                    the FP32 walk without rich tallies, 256 otherwise.
-                                   0: 256, or 512 (384 with continuum or excitation
-                                   tallies) in FP32 runs of profile mode 2 without
-                                   per-segment tallies that have many packets      */
+                                   Shared memory holds two CTAs per SM at any size,
+                                   so less than 256 leaves warps unused.
+                                   0, FP32 runs of profile mode 2 without mean
+                                   intensity or emissivity, tables in shared memory:
+                                   256 (the same form of the walk as 256 here), or
+                                   with at least 1024 packets per SM 512 (384 with
+                                   any rich tally, collisions or continuum).
+                                   0, all other runs: the largest size allowed       */
     int ctas_per_sm;            /* resident CTAs per SM of the persistent grid      */
     int refill_min;             /* a warp takes new packets once at least this many
                                    of its lanes are idle (1..32); 0: the walk

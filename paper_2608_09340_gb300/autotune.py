@@ -10,6 +10,9 @@ from __future__ import annotations
 
 import itertools
 
+# (An untuned run, block 0 and refill 0, chooses both for itself, with many
+# packets of a line with excitation or continuum a CTA of 384 threads that
+# cannot be asked for: pass a space with 0 in both lists to have that tried.)
 DEFAULT_SPACE = {
     "block": (256, 512),
     "refill_min": (1, 4, 16),

@@ -418,7 +418,7 @@ krl_status resolve_tune(const krl_tune* tune, krl_tune& T)
     }
     if (T.block && (T.block < 32 || T.block > 512 || T.block % 32))
         return fail(KRL_ERR_ARG, "block must be a multiple of 32 in [32, 512]");
-    if (T.refill_min < 0 || T.refill_min > 32) return fail(KRL_ERR_ARG, "refill_min must be in [1, 32]");
+    if (T.refill_min < 0 || T.refill_min > 32) return fail(KRL_ERR_ARG, "refill_min must be in [0, 32]");
     return KRL_OK;
 }
 
@@ -732,7 +732,9 @@ krl_status krl_run_packets(krl_grid* g, uint64_t n, uint64_t first_id, uint64_t 
     // 14.4 / 32.2.
     if (!(f & F_SEG) && mode == 2 && T.precision == KRL_PREC_FP32) {
         if (T.block) {
-            if (!(f & F_RICH)) f |= F_WIDE;     // the lean walk takes any CTA up to 512
+            // (the lean walk takes any CTA up to 512; at 256 and below the form
+            // with more registers has as many CTAs per SM)
+            if (!(f & F_RICH) && T.block > 256) f |= F_WIDE;
         } else if (n >= 2ull * 2ull * 256ull * (unsigned)g->num_sms) {
             f |= F_WIDE;
             T.block = transport_wide_block(f);
