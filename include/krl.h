@@ -24,8 +24,8 @@
  *  - Device memory comes from two memory pools of the library's own per device
  *    (grids and batches; scratch of a call). Of what they do not use they keep
  *    at most 256 MiB and 6 GiB mapped across synchronisations; the scratch
- *    pool is emptied with the device's last grid, and both before an
- *    allocation is reported as failed.
+ *    pool is emptied with the device's last grid, and both, after a wait for
+ *    the device, before an allocation is reported as failed.
  *  - Every call is ordered on the caller's stream `s` (a cudaStream_t; NULL
  *    is the legacy default stream). A call synchronises `s` only when it
  *    returns host data (documented per call).

@@ -12,6 +12,7 @@
 #include <mutex>
 #include <vector>
 
+#include "device_pools.cuh"
 #include "krl_internal.cuh"
 
 using namespace krl;
@@ -102,68 +103,6 @@ krl_status cuda_fail(cudaError_t e, const char* what)
         cudaError_t e_ = (call);                      \
         if (e_ != cudaSuccess) return cuda_fail(e_, what); \
     } while (0)
-
-// Device memory comes from two stream-ordered pools of the library's own per
-// device, one for what grids and batches keep, one for the scratch of a call,
-// so that creating, replacing and destroying lines, and calls that the caller
-// waits for, do not map and unmap memory each time: a synchronisation unmaps
-// what a pool holds unused above its threshold, with the default pool all of
-// it (7 ms of a 27 ms ray trace with 4.3 GB of scratch). The thresholds bound
-// what stays mapped; with the device's last grid the scratch pool is emptied.
-struct DevicePools {
-    cudaMemPool_t kept = nullptr, scratch = nullptr;
-    int grids = 0;
-};
-constexpr unsigned long long kKeptIdle = 256ull << 20, kScratchIdle = 6ull << 30;
-constexpr int kMaxDevices = 64;
-std::mutex g_pool_mu;
-DevicePools g_pools[kMaxDevices];
-
-cudaError_t make_pool(int dev, unsigned long long idle, cudaMemPool_t* out)
-{
-    cudaMemPoolProps p{};
-    p.allocType = cudaMemAllocationTypePinned;
-    p.location.type = cudaMemLocationTypeDevice;
-    p.location.id = dev;
-    cudaError_t e = cudaMemPoolCreate(out, &p);
-    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(*out, cudaMemPoolAttrReleaseThreshold, &idle);
-    return e;
-}
-
-// The current device's pools, made on first use. grids: change of its count
-// of grids.
-cudaError_t device_pools(DevicePools* out, int grids = 0)
-{
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(g_pool_mu);
-    DevicePools& P = g_pools[dev];
-    if (!P.kept) e = make_pool(dev, kKeptIdle, &P.kept);
-    if (e == cudaSuccess && !P.scratch) e = make_pool(dev, kScratchIdle, &P.scratch);
-    P.grids += grids;
-    *out = P;
-    return e;
-}
-
-// From one of the pools, in the order of s; when there is no memory, once more
-// after unmapping what both hold unused.
-cudaError_t pool_alloc(void** p, size_t bytes, bool scratch, cudaStream_t s)
-{
-    DevicePools P;
-    cudaError_t e = device_pools(&P);
-    if (e != cudaSuccess) return e;
-    const cudaMemPool_t pool = scratch ? P.scratch : P.kept;
-    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    if (e == cudaErrorMemoryAllocation) {
-        (void)cudaGetLastError();
-        (void)cudaMemPoolTrimTo(P.kept, 0);
-        (void)cudaMemPoolTrimTo(P.scratch, 0);
-        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    }
-    return e;
-}
 
 // Kept memory: usable on every stream once s has been synchronised (each call
 // that allocates does so), and freed when nothing on the device uses it.
