@@ -25,7 +25,8 @@
  *    (grids and batches; scratch of a call). Of what they do not use they keep
  *    at most 256 MiB and 6 GiB mapped across synchronisations; the scratch
  *    pool is emptied with the device's last grid, and both, after a wait for
- *    the device, before an allocation is reported as failed.
+ *    the device, before an allocation is reported as failed. Another
+ *    allocator of the process gets that memory with krl_memory_trim.
  *  - Every call is ordered on the caller's stream `s` (a cudaStream_t; NULL
  *    is the legacy default stream). A call synchronises `s` only when it
  *    returns host data (documented per call).
@@ -69,6 +70,10 @@ KRL_API const char* krl_last_error(void);
 
 /* Library version, major * 10000 + minor * 100 + patch. */
 KRL_API int krl_version(void);
+
+/* Gives back the memory that the library's pools on the current device hold
+ * unused (see above); waits for the device. */
+KRL_API krl_status krl_memory_trim(void);
 
 /* ------------------------------------------------------------------ grid */
 

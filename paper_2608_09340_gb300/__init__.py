@@ -121,7 +121,7 @@ assert RECORD_DTYPE.itemsize == 24
 EXPORTS = ["krl_last_error", "krl_version", "krl_grid_create", "krl_grid_destroy", "krl_line_set",
            "krl_line_info_get", "krl_run_packets", "krl_tallies_get", "krl_tally_bytes", "krl_tallies_reset",
            "krl_emission_cdf_noalloc", "krl_raytrace_channels", "krl_batch_create", "krl_batch_run",
-           "krl_batch_destroy", "krl_levels_solve", "krl_levels_iterate"]
+           "krl_batch_destroy", "krl_levels_solve", "krl_levels_iterate", "krl_memory_trim"]
 
 _lib_handle = None
 
@@ -161,7 +161,7 @@ def load_library(path: str | None = None):
     for name in ("krl_grid_create", "krl_grid_destroy", "krl_line_set", "krl_line_info_get",
                  "krl_run_packets", "krl_tallies_get", "krl_tallies_reset", "krl_emission_cdf_noalloc",
                  "krl_raytrace_channels", "krl_batch_create", "krl_batch_destroy", "krl_batch_run",
-                 "krl_levels_solve", "krl_levels_iterate"):
+                 "krl_levels_solve", "krl_levels_iterate", "krl_memory_trim"):
         getattr(lib, name).restype = C.c_int
     if path is None:
         _lib_handle = lib
@@ -235,6 +235,12 @@ def krl_tallies_reset(handle, stream=None):
 
 def krl_raytrace_channels(handle, desc: krl_raytrace_desc, maps, stream=None):
     _check(load_library().krl_raytrace_channels(handle, C.byref(desc), _ptr(maps), _stream_handle(stream)))
+
+
+def krl_memory_trim():
+    """Gives back the device memory that the library holds unused, up to 6.25
+    GiB, to be had by PyTorch's allocator; waits for the device."""
+    _check(load_library().krl_memory_trim())
 
 
 def krl_emission_cdf_noalloc(rate, cdf, stream=None):

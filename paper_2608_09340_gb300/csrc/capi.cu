@@ -377,6 +377,12 @@ const char* krl_last_error(void) { return g_err; }
 
 int krl_version(void) { return 500; }       // 0.5.0: records carry scat_cells; krl_tune.table_space
 
+krl_status krl_memory_trim(void)
+{
+    KRL_CUDA(pools_trim(), "krl_memory_trim");
+    return KRL_OK;
+}
+
 krl_status krl_grid_create(krl_grid** out, const krl_grid_desc* d, krl_stream st)
 {
     cudaStream_t s = (cudaStream_t)st;

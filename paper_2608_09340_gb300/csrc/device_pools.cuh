@@ -78,4 +78,16 @@ inline cudaError_t pool_alloc(void** p, size_t bytes, bool scratch, cudaStream_t
     return e;
 }
 
+// Unmaps what the current device's pools hold unused, what is being freed
+// behind work in flight included.
+inline cudaError_t pools_trim()
+{
+    DevicePools P;
+    cudaError_t e = device_pools(&P);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemPoolTrimTo(P.kept, 0);
+    if (e == cudaSuccess) e = cudaMemPoolTrimTo(P.scratch, 0);
+    return e;
+}
+
 }  // namespace krl

@@ -51,6 +51,11 @@ int main(int argc, char** argv)
     pending = held;                 // freed behind work in flight
     capturing = cap;
     calls.clear();
+    if (argc > 5) {
+        const cudaError_t t = pools_trim();
+        printf("%d %s%zu\n", (int)t, calls.c_str(), room);
+        return 0;
+    }
     const cudaError_t e = pool_alloc(&p, want, scratch, nullptr);
     printf("%d %s\n", (int)e, calls.c_str());
     return 0;
@@ -67,8 +72,9 @@ def alloc(tmp_path_factory):
     subprocess.check_call(["g++", "-std=c++17", "-I", os.path.join(CUDA, "include"), "-I",
                            os.path.join(ROOT, "paper_2608_09340_gb300", "csrc"), str(d / "p.cpp"), "-o", str(d / "p")])
 
-    def run(scratch, capturing, held, want):
-        out = subprocess.check_output([str(d / "p"), str(int(scratch)), str(int(capturing)), str(held), str(want)], text=True)
+    def run(scratch, capturing, held, want, *trim):
+        args = [str(int(v)) for v in (scratch, capturing, held, want, *trim)]
+        out = subprocess.check_output([str(d / "p"), *args], text=True)
         e, calls = out.split()
         return int(e), calls
     return run
@@ -89,3 +95,7 @@ def test_kept_memory_that_is_not_there(alloc):
 def test_scratch_and_captures_do_not_wait(alloc):
     assert alloc(True, False, 80, 50) == (2, "atta")
     assert alloc(False, True, 80, 50) == (2, "atta")
+
+
+def test_trim_gives_everything_back(alloc):
+    assert alloc(False, False, 80, 0, 1) == (0, "wtt100")
