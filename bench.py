@@ -191,7 +191,7 @@ RT_CHANNELS = 64
 RT_PIXELS = 1024
 RT_CAMERAS = 3
 RT_PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "raytrace_envelope128_64ch.txt")
-RT_KERNEL_SRC = [os.path.join(ROOT, "paper_2608_09340_gb300", "csrc", f) for f in ("raytrace.cu", "krl_internal.cuh")]
+RT_KERNEL_SRC = [os.path.join(ROOT, "paper_2608_09340_gb300", "csrc", f) for f in ("raytrace.cu", "krl_internal.cuh", "trace_tile.cuh")]
 # Arithmetic of one channel-segment of the formal solution (Eq. imaging-
 # formal): dtau = alpha dl, e = exp(-dtau), f = (1 - e)/dtau (2), the
 # increment T j dl f (3), I += it, tau += dtau, T = exp(-tau): 10 ops.

@@ -15,11 +15,13 @@
 // the imaging pass as the two-step scheme does (Sec. 3.2).
 //
 // GPU layout: per camera, a prep kernel tabulates the channel extinction
-// alpha_k per (cell, channel) (it depends on the cell and the channel only);
-// the trace then gives each ray a group of lanes with the channels across
-// them (4 per lane), so that a cell's [n_ch] rows are coalesced reads and a
-// warp follows several neighbouring rays. Without memory for the cube, one
-// warp per pixel evaluates the profile per segment. Rays are marched from
+// alpha_k per (cell, channel) (it depends on the cell and the channel only)
+// and the trace reads it, in one of two layouts (launch_trace_any chooses): a
+// warp's lanes follow 32 neighbouring pixels' rays, each over the same 1 to 8
+// channels (k_trace_cube; the usual one), or 4 to 32 lanes share a ray, 4
+// channels each, so that a cell's [n_ch] rows are coalesced reads
+// (k_trace_rows; few or widely spaced pixels). Without memory for the cube,
+// one warp per pixel evaluates the profile per segment. Rays are marched from
 // the camera side backwards; each channel sums
 // I = sum_seg T j dl f(dtau) with T = exp(-tau in front of the segment), the
 // optical depth and the sum carried with compensated (Kahan) addition so

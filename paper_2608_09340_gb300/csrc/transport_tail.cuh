@@ -18,7 +18,8 @@
 // packet) marks how many of the scatterings stand; the rest are walked again
 // from the next cell, with the same draws. A packet alone then takes 150 to
 // 200 ns per event (690 to 1000 before): 1e5 packets in the outflowing sphere
-// 938 -> 396 ms, 1e4 in the slab 138 -> 33 ms, together with the other steps.
+// 938 -> 389 ms, 1e4 in the slab 143 -> 35.5 ms (183 -> 44 with the packets
+// of another seed), together with the other steps.
 //
 // Every value is formed by the functions and in the order of advance(), so a
 // packet continues bit for bit as it would have in a lane of its own.
@@ -31,8 +32,9 @@
 // and a CTA with few packets above kTailWide rather waits for some to end.
 // Measured with both / with groups of 8 only, means of three seeds: outflow of
 // 1e5 packets 368 / 369 ms, static sphere 492 / 500, dusty slab 107 / 109,
-// 64 models 162 / 167, 1e4-packet slab 35.8 / 35.1; with groups of 4 from
-// 2 kTailWide down the slab (33 packets per CTA) took 52 for 44.
+// 64 models 162 / 167, 1e4-packet slab 35.8 / 35.1 (all but the models'
+// within the scatter of these calls); with groups of 4 from 2 kTailWide down
+// the slab (33 packets per CTA) took 52 for 44 with a fourth seed's packets.
 //
 // Runs with an emissivity tally (TransportArgs::tail_warps) use kTailWarpsL1:
 // a segment that the walk deposits itself reads the R_IIA table through L1,
