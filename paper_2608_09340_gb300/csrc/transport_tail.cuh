@@ -43,7 +43,7 @@
 // runs, without groups (17 KB for the stash) / 8 warps / 6: 128^3 envelope, 3
 // cameras x 64 channels, 1e6 packets deposited in the walk 20.3 / 27.0 / 22.0
 // ms, 4e6 with the default buffer 46.9 / 52.3 / 46.1, a box of tau0 = 100 with
-// 1e5 packets 32.3 / 40.7 / 33.4. Without that tally 8 are better (box of
+// 1e5 packets 32.5 / 41.1 / 31.8. Without that tally 8 are better (box of
 // tau0 = 1000 with mean intensity, 1e5 packets: 27.0 / 12.5 / 13.4).
 //
 // With the tables in the constant bank (mode 4) the lanes of a group read
@@ -434,25 +434,26 @@ __device__ __forceinline__ void walk_tail(const TransportArgs& A, const RoundKey
             return ((bits >> s0) | (s0 ? bits << (G - s0) : 0u)) & group;
         };
         stop = order(stop);
-        // A scattering without its row still has its own profile and place, so
-        // a crossing, absorption or destruction there stands, its outcome does
+        // A scattering without its row has its own profile and place: a
+        // crossing, absorption or destruction there stands, its outcome does
         // not. The place after one beyond |x| = 300 was evaluated with another
-        // frequency than the packet has: nothing from there on stands.
-        unsigned lost = 0u, wrong = 0u;
+        // frequency than the packet has: whether it stops there is not known.
+        unsigned lost = 0u;
         if (__any_sync(kFull, pos < now && (out || far))) {     // rare
             lost = order(__ballot_sync(kFull, pos < now && out) >> base);
-            wrong = order(__ballot_sync(kFull, pos < now && far) >> base) << 1;
+            const unsigned wrong = order(__ballot_sync(kFull, pos < now && far) >> base) << 1;
+            stop &= ~wrong;
+            lost |= wrong;
         }
         int lim = room < (uint32_t)now ? (int)room : now;
-        const int fo = lost ? __ffs(lost) - 1 : 64, fw = wrong ? __ffs(wrong) - 1 : 64;
+        const int fo = lost ? __ffs(lost) - 1 : 64;
         int f = stop ? __ffs(stop) - 1 : now;
-        if (fw < lim) lim = fw;
         const bool ends = f < lim && f <= fo;           // segment f runs, and is not a plain scattering
         if (fo < lim) lim = fo;
         f = alive ? (f < lim ? f : lim) : 0;            // (a group without a packet keeps known >= 0)
         have -= f;
         known -= f;
-        if (!ends && (f == fo || f == fw)) {            // draw again, the window around x
+        if (!ends && f == fo) {                         // draw again, the window around x
             have = known = 0;
             ev = 0;
         }
