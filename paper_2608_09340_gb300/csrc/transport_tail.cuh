@@ -44,7 +44,9 @@
 // cameras x 64 channels, 1e6 packets deposited in the walk 20.3 / 27.0 / 22.0
 // ms, 4e6 with the default buffer 46.9 / 52.3 / 46.1, a box of tau0 = 100 with
 // 1e5 packets 32.5 / 41.1 / 31.8. Without that tally 8 are better (box of
-// tau0 = 1000 with mean intensity, 1e5 packets: 27.0 / 12.5 / 13.4).
+// tau0 = 1000 with mean intensity, 1e5 packets: 27.0 / 12.5 / 13.4). The 32
+// packets of one warp's draw of ids, a CTA's all in a run of few, are among
+// those that 6 warps start with in groups of 4.
 //
 // With the tables in the constant bank (mode 4) the lanes of a group read
 // different addresses, which that bank serves one after the other, so that
@@ -56,7 +58,7 @@ constexpr int kTailWarps = 8, kTailWarpsL1 = 6, kTailWarpsConst = 4;
 constexpr int kTailWide = 4;
 constexpr bool tail_starts(int total, int warps)
 {
-    return total <= warps * kTailWide || (total <= warps * 2 * kTailWide && 3 * total > warps * 4 * kTailWide);
+    return total <= warps * kTailWide || (total <= warps * 2 * kTailWide && 3 * total >= warps * 4 * kTailWide);
 }
 
 // Rows inverted ahead (odd: no bank conflicts between slots). In the line's
